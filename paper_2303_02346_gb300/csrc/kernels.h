@@ -152,8 +152,15 @@ void launch_mass_loss_grad(const Params& P, const float* st, const uint32_t* tag
 // grid-stride kernels size their grids as a multiple of it
 int sm_count();
 void launch_init_state(float* st, int N, cudaStream_t s);
-void launch_init_particles(float* X0, uint32_t* tag0, const uint8_t* mat, int lo, int cnt, int N,
-                           int n_mat, int* err, cudaStream_t s);
+// Particles [lo, lo + cnt) of the initial state (SoA, N stride) from caller rows
+// x, v [cnt][3] and material indices: C = 0, F = I, material tags.
+void launch_init_particles(float* X0, uint32_t* tag0, const float* x, const float* v, const uint8_t* mat, int lo,
+                           int cnt, int N, int n_mat, int* err, cudaStream_t s);
+// Particles [lo, lo + cnt) (caller order) of the SoA state `st`, whose particle
+// p is the caller's pid[p] (nullptr: p), into rows x, v [cnt][3], C, F [cnt][9]
+// (each nullable); a liquid's F is diag(J, 1, 1). tag0: tags in caller order.
+void launch_read_state(const Params& P, const float* st, const uint32_t* tag0, const int* pid, int lo, int cnt,
+                       float* x, float* v, float* C, float* F, cudaStream_t s);
 void launch_iota(int* a, int N, cudaStream_t s);
 // dst[i] += src[i] for i < n; with clear_src also src[i] = 0
 void launch_add_fields(float* dst, float* src, long long n, int clear_src, cudaStream_t s);

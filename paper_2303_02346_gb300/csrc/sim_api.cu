@@ -130,6 +130,9 @@ struct mpm_sim {
   float *lm = nullptr, *ltm = nullptr, *ltd = nullptr, *ldm = nullptr;
   double* dloss = nullptr;
   int* err = nullptr;
+  // pinned copies of device words, so that one synchronisation of the stream
+  // brings them to the host: [0] = err, [1] = nwater, [2] = ovf
+  int* words = nullptr;
   // first of the horizon's last chunks whose per-step data (states, grids,
   // SVDs) the forward that reached max_steps left in the chunk buffers (chunk
   // c in buffer n_ckpt - 1 - c); a backward over that horizon sweeps them
@@ -377,14 +380,17 @@ void do_sort(sim_h h, const float* st_in, const uint32_t* tag_in, const int* pid
   h->launches += h->P.N > 0 ? 5 : 3;
 }
 
+// Wait for the stream and read the error word. The word is copied to pinned
+// memory on the stream before the wait: a second, blocking copy after it
+// costs another round trip to the device (about 10 us a call).
 sim_status check_err(sim_h h, const char* where) {
-  cudaError_t e = cudaStreamSynchronize(h->stream);
+  cudaError_t e = cudaMemcpyAsync(h->words, h->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  const cudaError_t es = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess) e = es;
   if (e != cudaSuccess) return cuda_fail(h, e, where);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, where);
-  int flag = 0;
-  e = cudaMemcpy(&flag, h->err, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(h, e, where);
+  const int flag = h->words[0];
   // a particle that leaves the grid is the usual root cause of later non-finite values
   if (flag & kErrDomain)
     return fail(h, SIM_E_DOMAIN, std::string(where) + ": a particle's stencil left the grid");
@@ -929,6 +935,7 @@ sim_status sim_destroy(sim_h h) {
   if (h->ev_join) cudaEventDestroy(h->ev_join);
   if (h->rstream) cudaStreamDestroy(h->rstream);
   if (h->hstream) cudaStreamDestroy(h->hstream);
+  if (h->words) cudaFreeHost(h->words);
   delete h;
   return SIM_OK;
 }
@@ -1002,7 +1009,8 @@ sim_status sim_create(const sim_config* c, sim_h* out) {
             dalloc(h, &h->flags, h->nflags) && dalloc(h, &h->list, 2 * h->nflags) &&
             dalloc(h, &h->count, 2) && dalloc(h, &h->err, 1) && dalloc(h, &h->dloss, h->S) &&
             dalloc(h, &h->tile_ctr, 2) && dalloc(h, &h->bar, 2) && dalloc(h, &h->nwater, 1) &&
-            dalloc(h, &h->rows, (size_t)N * kStateFields) && dalloc(h, &h->inv, N);
+            dalloc(h, &h->rows, (size_t)N * kStateFields) && dalloc(h, &h->inv, N) &&
+            cudaMallocHost(&h->words, 3 * sizeof(int)) == cudaSuccess;
   h->sb.n_bins = int(nbins);
   ok = ok && dalloc(h, &h->sb.key, N) && dalloc(h, &h->sb.rank, N) && dalloc(h, &h->sb.bins, 2 * nbins + 1) &&
        dalloc(h, &h->sb.tile_sums, 2 * nbins / 4096 + 2);
@@ -1035,6 +1043,7 @@ sim_status sim_create(const sim_config* c, sim_h* out) {
     }
   }
   if (!ok) {
+    cudaGetLastError();
     sim_destroy(h);
     return SIM_E_OOM;
   }
@@ -1082,19 +1091,26 @@ sim_status sim_set_particles(sim_h h, int scene, const float* x, const float* v,
   if (!scene_range(h, scene, &lo, &cnt)) return fail(h, SIM_E_ARG, "sim_set_particles: bad scene");
   if (cnt > 0 && (!x || !v || !mat)) return fail(h, SIM_E_ARG, "sim_set_particles: null pointer");
   const int N = h->N;
-  // staging in the N x 24 rows buffer: x at 0, v at 3N, material bytes at 6N
-  float* stage = h->rows;
-  uint8_t* mstage = reinterpret_cast<uint8_t*>(stage + (size_t)6 * N);
-  cudaError_t e = to_device(h, stage, x, sizeof(float) * 3 * cnt, on_device);
-  if (e == cudaSuccess) e = to_device(h, stage + (size_t)3 * N, v, sizeof(float) * 3 * cnt, on_device);
-  if (e == cudaSuccess) e = to_device(h, mstage, mat, cnt, on_device);
-  if (e != cudaSuccess) return cuda_fail(h, e, "sim_set_particles");
+  // host arrays are staged in the N x 24 rows buffer (x at 0, v at 3N,
+  // material bytes at 6N); device arrays are read where they are
+  const float *xs = x, *vs = v;
+  const uint8_t* ms = mat;
+  cudaError_t e = cudaSuccess;
+  if (!on_device) {
+    float* stage = h->rows;
+    uint8_t* mstage = reinterpret_cast<uint8_t*>(stage + (size_t)6 * N);
+    e = to_device(h, stage, x, sizeof(float) * 3 * cnt, 0);
+    if (e == cudaSuccess) e = to_device(h, stage + (size_t)3 * N, v, sizeof(float) * 3 * cnt, 0);
+    if (e == cudaSuccess) e = to_device(h, mstage, mat, cnt, 0);
+    if (e != cudaSuccess) return cuda_fail(h, e, "sim_set_particles");
+    xs = stage;
+    vs = stage + (size_t)3 * N;
+    ms = mstage;
+  }
   cudaMemsetAsync(h->err, 0, sizeof(int), h->stream);
   // rows -> SoA fields of X0 at [lo, lo + cnt); C = 0, F = I, material tags
-  launch_gather_rows(stage, h->X0 + lo, nullptr, cnt, 3, 0, N, 0, h->stream);
-  launch_gather_rows(stage + (size_t)3 * N, h->X0 + (size_t)3 * N + lo, nullptr, cnt, 3, 0, N, 0, h->stream);
-  launch_init_particles(h->X0, h->tag0, mstage, lo, cnt, N, h->cfg.n_materials, h->err, h->stream);
-  h->launches += cnt > 0 ? 3 : 0;
+  launch_init_particles(h->X0, h->tag0, xs, vs, ms, lo, cnt, N, h->cfg.n_materials, h->err, h->stream);
+  h->launches += cnt > 0 ? 1 : 0;
   // water / other materials split of all scenes (the sort puts the water first)
   launch_count_water(h->P, h->tag0, h->nwater, h->stream);
   h->launches += N > 0 ? 1 : 0;
@@ -1103,11 +1119,13 @@ sim_status sim_set_particles(sim_h h, int scene, const float* x, const float* v,
     launch_rigid_rest(h->P, h->X0, h->tag0, scene, lo, cnt, h->rb, h->stream);
     h->launches += cnt > 0 ? 4 : 0;
   }
-  int flag = 0, nw = 0;
-  e = cudaStreamSynchronize(h->stream);
-  if (e == cudaSuccess) e = cudaMemcpy(&flag, h->err, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) e = cudaMemcpy(&nw, h->nwater, sizeof(int), cudaMemcpyDeviceToHost);
+  e = cudaMemcpyAsync(h->words, h->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(h->words + 1, h->nwater, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  const cudaError_t es = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess) e = es;
   if (e != cudaSuccess) return cuda_fail(h, e, "sim_set_particles");
+  const int flag = h->words[0], nw = h->words[1];
   if (flag & kErrArg) {
     h->initialized = false;
     return fail(h, SIM_E_ARG, "sim_set_particles: material index out of range");
@@ -1120,7 +1138,10 @@ sim_status sim_set_particles(sim_h h, int scene, const float* x, const float* v,
   }
   restart(h);
   h->initialized = true;
-  return check_err(h, "sim_set_particles");
+  // the caller's arrays were read before the synchronisation above; the
+  // restart's copies and clears are left to the stream
+  e = cudaGetLastError();
+  return e == cudaSuccess ? SIM_OK : cuda_fail(h, e, "sim_set_particles");
 }
 
 sim_status sim_set_state(sim_h h, int scene, const float* x, const float* v, const float* C, const float* F,
@@ -1182,9 +1203,10 @@ int sim_current_step(sim_h h) { return h ? h->step : -1; }
 // every earlier one are left to the backward's recompute.
 static sim_status drop_overflowed_chunks(sim_h h) {
   if (!h->ovf || h->rec_from < 0 || h->rec_from >= h->n_ckpt) return SIM_OK;
-  int bits = 0;
-  cudaError_t e = cudaMemcpy(&bits, h->ovf, sizeof(int), cudaMemcpyDeviceToHost);
+  cudaError_t e = cudaMemcpyAsync(h->words + 2, h->ovf, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "sim_step");
+  const int bits = h->words[2];
   int from = h->rec_from;
   for (int c = h->rec_from; c < h->n_ckpt; ++c) {
     const int b = h->n_ckpt - 1 - c;
@@ -1298,43 +1320,29 @@ sim_status sim_get_state(sim_h h, int scene, int step, float* x, float* v, float
                 "sim_get_state: the state of step " + std::to_string(t) +
                     " is not retained (retained: step 0, the current step and the checkpoint steps before it)");
   }
-  // rows (caller layout, all particles): x3 v3 C9 F9 per particle
-  launch_gather_rows(src, h->rows, pid, N, kStateFields, N, 0, 1, h->stream);
-  h->launches += N > 0 ? 1 : 0;
-  std::vector<float> host;
-  std::vector<uint32_t> tags;
-  if (cudaStreamSynchronize(h->stream) != cudaSuccess) return cuda_fail(h, cudaGetLastError(), "sim_get_state");
-  host.resize((size_t)cnt * kStateFields);
-  tags.resize(cnt);
-  cudaError_t e = cudaMemcpy(host.data(), h->rows + (size_t)lo * kStateFields,
-                             sizeof(float) * host.size(), cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess && cnt) e = cudaMemcpy(tags.data(), h->tag0 + lo, sizeof(uint32_t) * cnt, cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(h, e, "sim_get_state");
-  std::vector<float> ox(x ? 3 * (size_t)cnt : 0), ov(v ? 3 * (size_t)cnt : 0), oC(C ? 9 * (size_t)cnt : 0),
-      oF(F ? 9 * (size_t)cnt : 0);
-  for (int i = 0; i < cnt; ++i) {
-    const float* r = host.data() + (size_t)i * kStateFields;
-    bool liquid = is_liquid(h->P.mat[tag_mat(tags[i])].kind);
-    for (int c = 0; c < 3; ++c) {
-      if (x) ox[3 * i + c] = r[c];
-      if (v) ov[3 * i + c] = r[3 + c];
-    }
-    for (int c = 0; c < 9; ++c) {
-      if (C) oC[9 * i + c] = r[6 + c];
-      if (F) oF[9 * i + c] = liquid ? (c == 0 ? r[15] : ((c % 4 == 0) ? 1.0f : 0.0f)) : r[15 + c];
+  // one pass from the state's own order to the caller's rows: straight into
+  // device outputs, through the rows buffer for host ones
+  float* host[4] = {x, v, C, F};
+  const int nc[4] = {3, 3, 9, 9};
+  float* dev[4] = {x, v, C, F};
+  if (!on_device) {
+    size_t off = 0;
+    for (int q = 0; q < 4; ++q) {
+      dev[q] = host[q] ? h->rows + off : nullptr;
+      off += (size_t)nc[q] * cnt;
     }
   }
-  struct {
-    float* dst;
-    std::vector<float>* src;
-  } outs[4] = {{x, &ox}, {v, &ov}, {C, &oC}, {F, &oF}};
-  for (auto& o : outs) {
-    if (!o.dst) continue;
-    e = on_device ? cudaMemcpy(o.dst, o.src->data(), sizeof(float) * o.src->size(), cudaMemcpyHostToDevice)
-                  : (std::memcpy(o.dst, o.src->data(), sizeof(float) * o.src->size()), cudaSuccess);
-    if (e != cudaSuccess) return cuda_fail(h, e, "sim_get_state");
+  if (x || v || C || F) {
+    launch_read_state(h->P, src, h->tag0, pid, lo, cnt, dev[0], dev[1], dev[2], dev[3], h->stream);
+    h->launches += N > 0 && cnt > 0 ? 1 : 0;
   }
-  return SIM_OK;
+  cudaError_t e = cudaGetLastError();
+  for (int q = 0; q < 4 && !on_device && e == cudaSuccess; ++q)
+    if (host[q] && cnt)
+      e = cudaMemcpyAsync(host[q], dev[q], sizeof(float) * nc[q] * cnt, cudaMemcpyDeviceToHost, h->stream);
+  const cudaError_t es = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess) e = es;
+  return e == cudaSuccess ? SIM_OK : cuda_fail(h, e, "sim_get_state");
 }
 
 sim_status sim_get_tool_pose(sim_h h, int scene, int step, float* pose, int on_device) {
