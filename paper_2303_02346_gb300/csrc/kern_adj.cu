@@ -114,38 +114,14 @@ __device__ inline void g2p_adj_gather(const Params& P, int p, const MatParams& M
     xb[d] += P.inv_dx * (xs[d] - (Cq[d] * Gv[0] + Cq[3 + d] * Gv[1] + Cq[6 + d] * Gv[2]));
 }
 
-// Scatter part of the G2P adjoint (every thread must call it):
+// Scatter part of the G2P adjoint (every lane must call it):
 // vbar_i += W (u + Cq o) for the node at stencil offset o.
 template <int NT>
-__device__ inline void g2p_adj_scatter(ScatterTile<NT>& T, const Params& P, bool valid, int scene,
+__device__ inline void g2p_adj_scatter(ScatterSmem<NT>& T, const Params& P, bool valid, int scene,
                                        const Stencil& sc, const float* u, const float* Cq,
                                        float4* __restrict__ gadj_v) {
-  scatter_setup(T, valid, sc.base, scene);
-  if (T.box[7]) {
-    const int rank = scatter_count(T, valid, sc.base);
-    __syncthreads();
-    scan_cells(T);
-    if (valid) scatter_record_affine(T, rank, sc, 0.0f, u, Cq);
-    __syncthreads();
-    scatter_accumulate<false, NT>(T);
-  } else if (valid) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const float W = sc.w[0][a] * sc.w[1][b] * sc.w[2][c];
-          float val[3];
-#pragma unroll
-          for (int i = 0; i < 3; ++i) val[i] = u[i] + float(a) * Cq[3 * i] + float(b) * Cq[3 * i + 1] + float(c) * Cq[3 * i + 2];
-          red_add_v4(gadj_v + node_index(P, scene, sc.base[0] + a, sc.base[1] + b, sc.base[2] + c),
-                     W * val[0], W * val[1], W * val[2], 0.0f);
-        }
-      }
-    }
-  }
-  scatter_flush(T, gadj_v, P, nullptr, nullptr, nullptr);
+  warp_scatter<false>(T.rec + (threadIdx.x & ~31) * kRecF4, P, valid, scene, sc, 0.0f, u, Cq, gadj_v, nullptr,
+                      nullptr, nullptr);
 }
 
 // kHigh: 4 resident CTAs of 256 per SM (64 registers) instead of 3
@@ -154,7 +130,7 @@ __global__ void __launch_bounds__(NT, (kHigh ? kScatterResidentThreadsHigh : kSc
 g2p_adj_kernel(Params P, const float* __restrict__ st_n, const float* __restrict__ st_n1,
                const uint32_t* __restrict__ tag, const float* __restrict__ Fp_n,
                float* __restrict__ adj, const float4* __restrict__ gv, float4* __restrict__ gadj_v) {
-  __shared__ ScatterTile<NT> T;
+  __shared__ ScatterSmem<NT> T;
   const int N = P.N;
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = p < N;
@@ -536,7 +512,7 @@ adj_fused_kernel(Params P, const float* __restrict__ st_prev, const float* __res
                  const float* __restrict__ svd_n, const float* __restrict__ Fp_prev,
                  float* __restrict__ adj, const float4* __restrict__ gadj_m,
                  const float4* __restrict__ gv_prev, float4* __restrict__ gadj_v) {
-  __shared__ ScatterTile<NT> T;
+  __shared__ ScatterSmem<NT> T;
   const int N = P.N;
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = p < N;
@@ -579,10 +555,11 @@ void launch_g2p_adj(const Params& P, const Tuning& tu, const float* st_n, const 
                     const uint32_t* tag, const float* Fp_n, float* adj, const float4* gv, float4* gadj_v,
                     cudaStream_t s) {
   if (P.N == 0) return;
-  if (tu.scatter_threads == 128) {
+  if (tu.scatter_threads == 128 && tu.scatter_ctas == 4) {
+    g2p_adj_kernel<128, true><<<blocks_for(P.N, 128), 128, 0, s>>>(P, st_n, st_n1, tag, Fp_n, adj, gv, gadj_v);
+  } else if (tu.scatter_threads == 128) {
     g2p_adj_kernel<128><<<blocks_for(P.N, 128), 128, 0, s>>>(P, st_n, st_n1, tag, Fp_n, adj, gv, gadj_v);
   } else if (tu.scatter_ctas == 4) {
-    max_shared_carveout(reinterpret_cast<const void*>(g2p_adj_kernel<256, true>));
     g2p_adj_kernel<256, true><<<blocks_for(P.N, 256), 256, 0, s>>>(P, st_n, st_n1, tag, Fp_n, adj, gv, gadj_v);
   } else {
     g2p_adj_kernel<256><<<blocks_for(P.N, 256), 256, 0, s>>>(P, st_n, st_n1, tag, Fp_n, adj, gv, gadj_v);

@@ -81,48 +81,20 @@ __device__ inline void p2g_prologue(const Params& P, int p, const MatParams& M, 
   if (!make_stencil(x, P, sc)) atomicOr(err, kErrDomain);
 }
 
-// Block-level scatter of the CTA's particles (every thread must call it).
+// Scatter of the warp's particles from their state in registers (every lane
+// must call it).
 template <int NT>
-__device__ inline void p2g_scatter(ScatterTile<NT>& T, const Params& P, bool valid, int scene,
+__device__ inline void p2g_scatter(ScatterSmem<NT>& T, const Params& P, bool valid, int scene,
                                    const Stencil& sc, float m, const float* v, const float* A,
                                    float4* __restrict__ acc, int* __restrict__ flags,
                                    int* __restrict__ list, int* __restrict__ count) {
-  scatter_setup(T, valid, sc.base, scene);
-  if (T.box[7]) {
-    // cell-binned tile: records sorted by cell, then per-(cell, o_x, o_y) accumulation
-    const int rank = scatter_count(T, valid, sc.base);
-    __syncthreads();
-    scan_cells(T);
-    if (valid) {
-      const float mv[3] = {m * v[0], m * v[1], m * v[2]};
-      scatter_record(T, rank, sc, m, mv, A, P.dx);
-    }
-    __syncthreads();
-    scatter_accumulate<true, NT>(T);
-  } else if (valid) {
-    const float mv0 = m * v[0], mv1 = m * v[1], mv2 = m * v[2];
+  float Md[9], cp[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const float da = (a - sc.f[0]) * P.dx;
+  for (int k = 0; k < 9; ++k) Md[k] = A[k] * P.dx;
 #pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const float db = (b - sc.f[1]) * P.dx;
-        const float wab = sc.w[0][a] * sc.w[1][b];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const float dc = (c - sc.f[2]) * P.dx;
-          const float W = wab * sc.w[2][c];
-          const float q0 = mv0 + A[0] * da + A[1] * db + A[2] * dc;
-          const float q1 = mv1 + A[3] * da + A[4] * db + A[5] * dc;
-          const float q2 = mv2 + A[6] * da + A[7] * db + A[8] * dc;
-          red_add_v4(acc + node_index(P, scene, sc.base[0] + a, sc.base[1] + b, sc.base[2] + c), W * m,
-                     W * q0, W * q1, W * q2);
-        }
-      }
-    }
-    mark_stencil_blocks(P, scene, sc.base, flags, list, count);
-  }
-  scatter_flush(T, acc, P, flags, list, count);
+  for (int i = 0; i < 3; ++i)
+    cp[i] = m * v[i] - (Md[3 * i] * sc.f[0] + Md[3 * i + 1] * sc.f[1] + Md[3 * i + 2] * sc.f[2]);
+  warp_scatter<true>(T.rec + (threadIdx.x & ~31) * kRecF4, P, valid, scene, sc, m, cp, Md, acc, flags, list, count);
 }
 
 // reset_count: the active-block counter of the other step parity (consumed by
@@ -133,7 +105,7 @@ p2g_kernel(Params P, const float* __restrict__ st, const uint32_t* __restrict__ 
            float* __restrict__ Fp_out, float* __restrict__ svd_out, float4* __restrict__ acc,
            int* __restrict__ flags, int* __restrict__ list, int* __restrict__ count,
            int* __restrict__ reset_count, int* __restrict__ err) {
-  __shared__ ScatterTile<NT> T;
+  __shared__ ScatterSmem<NT> T;
   const int N = P.N;
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p == 0 && reset_count) *reset_count = 0;
@@ -440,11 +412,16 @@ g2p_kernel(Params P, const float* __restrict__ st_in, float* __restrict__ st_out
 // Tensor-copy staging of the gather (kStage): the CTA reduces the bounding box
 // of its particles' G2P stencil origins; if the box's nodes fit in
 // kStageBox^3 and the particles share one scene, one thread issues a tiled
-// TMA load of that box of the previous step's grid velocities into the
-// scatter tile's accumulator storage (unused until the scatter), and the
-// gathers read shared memory instead of issuing 27 global loads a particle.
+// TMA load of that box of the previous step's grid velocities into shared
+// memory, and the gathers read there instead of issuing 27 global loads a
+// particle.
 template <int NT>
-__device__ inline bool stage_gather_box(ScatterTile<NT>& T, const Params& P, const CUtensorMap* gvmap, bool valid,
+struct alignas(128) StageSmem {
+  float4 box[kStageBox * kStageBox * kStageBox];
+  int red[2][4][NT / 32];
+};
+template <int NT>
+__device__ inline bool stage_gather_box(StageSmem<NT>& T, const Params& P, const CUtensorMap* gvmap, bool valid,
                                         const float* x, int scene, int* org, uint64_t* bar) {
   int b[3];
 #pragma unroll
@@ -487,7 +464,7 @@ __device__ inline bool stage_gather_box(ScatterTile<NT>& T, const Params& P, con
       sur::mbar_arrive_expect_tx(bar, kStageBox * kStageBox * kStageBox * 16);
       asm volatile(
           "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-          " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(sur::smem_u32(&T.acc[0][0])),
+          " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(sur::smem_u32(T.box)),
           "l"(reinterpret_cast<uint64_t>(gvmap)), "r"(0), "r"(mn[2]), "r"(mn[1]), "r"(mn[0]), "r"(mn[3]),
           "r"(sur::smem_u32(bar))
           : "memory");
@@ -511,7 +488,8 @@ g2p2g_kernel(Params P, const float* __restrict__ st_in, float* __restrict__ st_o
              float* __restrict__ svd_out, float4* __restrict__ acc, int* __restrict__ flags,
              int* __restrict__ list, int* __restrict__ count, int* __restrict__ reset_count,
              int* __restrict__ err, const __grid_constant__ CUtensorMap gvmap) {
-  __shared__ ScatterTile<NT> T;
+  __shared__ ScatterSmem<NT> T;
+  __shared__ StageSmem<kStage ? NT : 32> G;  // unused (and dropped) without kStage
   __shared__ uint64_t stage_bar;
   __shared__ int stage_org[4];
   const int N = P.N;
@@ -519,7 +497,7 @@ g2p2g_kernel(Params P, const float* __restrict__ st_in, float* __restrict__ st_o
   if (p == 0 && reset_count) *reset_count = 0;
   const bool valid = p < N;
   bool staged = false;
-  if (kStage) {
+  if constexpr (kStage) {
     float xs[3] = {0.f, 0.f, 0.f};
     int sc0 = 0;
     if (valid) {
@@ -527,7 +505,7 @@ g2p2g_kernel(Params P, const float* __restrict__ st_in, float* __restrict__ st_o
       for (int d = 0; d < 3; ++d) xs[d] = st_in[(fX + d) * N + p];
       sc0 = tag_scene(tag[p]);
     }
-    staged = stage_gather_box(T, P, &gvmap, valid, xs, sc0, stage_org, &stage_bar);
+    staged = stage_gather_box(G, P, &gvmap, valid, xs, sc0, stage_org, &stage_bar);
   }
   float x[3] = {0.f, 0.f, 0.f}, v[3] = {0.f, 0.f, 0.f}, A[9];
   float m = 0.0f;
@@ -542,7 +520,7 @@ g2p2g_kernel(Params P, const float* __restrict__ st_in, float* __restrict__ st_o
     float C[9], F[9];
     g2p_particle<kLean ? kStoreLean : kStoreChunk>(P, p, M, scene, st_in, st_out, Fp_prev, gv_prev, err, x, v,
                                                   C, F,
-                        staged ? reinterpret_cast<const float4*>(&T.acc[0][0]) : nullptr, stage_org,
+                        staged ? G.box : nullptr, stage_org,
                         &stage_bar);
     p2g_prologue<kExt>(P, p, M, x, C, F, Fp_out, svd_out, err, A, sc);
   }
@@ -608,7 +586,7 @@ __device__ inline bool grid_barrier(unsigned* bar, unsigned expected, int* err,
 // that its registers are allocated as in the per-step fused kernel, apart
 // from the run's loop state.
 template <int NT, bool kExt>
-__device__ __noinline__ void forward_tile(ScatterTile<NT>& T, const Params& P, int tile, int mode, const float* src,
+__device__ __noinline__ void forward_tile(ScatterSmem<NT>& T, const Params& P, int tile, int mode, const float* src,
                                           float* W, const uint32_t* __restrict__ tag, float* Fp, float4* acc,
                                           const float4* gv, int* flags, int* list, int* count, int* err) {
   const int N = P.N;
@@ -653,7 +631,7 @@ forward_run_kernel(Params P, const float* src, float* W, const uint32_t* __restr
                    float4* acc, float4* gv, int* flags, int* lists, long long list_stride, int* count,
                    const float* __restrict__ pose, int n0, int n1, int max_steps, int* tile_ctr, unsigned* bar,
                    int* err, unsigned long long timeout_ns) {
-  __shared__ ScatterTile<NT> T;
+  __shared__ ScatterSmem<NT> T;
   __shared__ int tile_sh[2];
   const int ntiles = (P.N + NT - 1) / NT;
   for (int n = n0; n < n1; ++n) {
@@ -666,7 +644,7 @@ forward_run_kernel(Params P, const float* src, float* W, const uint32_t* __restr
       tile_ctr[q ^ 1] = 0;
     }
     // tiles from the counter; thread 0 fetches the next tile's index while the
-    // CTA works on the current one (the tile's own barriers publish it)
+    // CTA works on the current one (the barrier after the tile publishes it)
     if (threadIdx.x == 0) tile_sh[0] = atomicAdd(tile_ctr + q, 1);
     __syncthreads();
     for (int it = 0;; ++it) {
@@ -675,6 +653,7 @@ forward_run_kernel(Params P, const float* src, float* W, const uint32_t* __restr
       if (threadIdx.x == 0) tile_sh[(it + 1) & 1] = atomicAdd(tile_ctr + q, 1);
       forward_tile<NT, kExt>(T, P, tile, n == n0 ? 0 : (n == n0 + 1 ? 1 : 2), src, W, tag, Fp, acc, gv, flags,
                              list, count + q, err);
+      __syncthreads();
     }
     if (!grid_barrier(bar, gridDim.x, err, timeout_ns)) return;
     int cnt;
@@ -716,6 +695,8 @@ void launch_p2g(const Params& P, const Tuning& tu, const float* st_in, const uin
 
 template <bool kLean, bool kStage>
 static auto g2p2g_variant(const Params& P, const Tuning& tu) {
+  if (tu.scatter_threads == 128 && tu.scatter_ctas == 4)
+    return P.ext ? g2p2g_kernel<128, true, kLean, kStage, true> : g2p2g_kernel<128, false, kLean, kStage, true>;
   if (tu.scatter_threads == 128)
     return P.ext ? g2p2g_kernel<128, true, kLean, kStage> : g2p2g_kernel<128, false, kLean, kStage>;
   if (tu.scatter_ctas == 4)
@@ -734,7 +715,6 @@ void launch_g2p2g(const Params& P, const Tuning& tu, const float* st_in, float* 
   auto k = lean ? (stage ? g2p2g_variant<true, true>(P, tu) : g2p2g_variant<true, false>(P, tu))
                 : (stage ? g2p2g_variant<false, true>(P, tu) : g2p2g_variant<false, false>(P, tu));
   const int nt = tu.scatter_threads == 128 ? 128 : 256;
-  if (nt == 256 && tu.scatter_ctas == 4) max_shared_carveout(reinterpret_cast<const void*>(k));
   CUtensorMap none;
   std::memset(&none, 0, sizeof(none));
   k<<<blocks_for(P.N, nt), nt, 0, s>>>(P, st_in, st_out, tag, Fp_prev, gv_prev, g.Fp, g.svd, g.acc, g.flags,

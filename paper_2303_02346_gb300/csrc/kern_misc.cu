@@ -2,8 +2,6 @@
 // between the library's particle order and the caller's, tool kinematics and
 // its adjoint, losses and loss seeds.
 #include <climits>
-#include <mutex>
-#include <set>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -19,8 +17,8 @@ static inline int blocks_for(long long n, int t) { return int((n + t - 1) / t); 
 // counting sort by (scene, Morton order of the cell of the stencil origin).
 // The Morton order keeps every 4^3 grid block contiguous (its cells are the
 // code's lowest 6 bits) and orders the particles of a block by cell, so that
-// a CTA's consecutive particles occupy few, densely filled cells: the scatter
-// tile then has fewer (cell, node) accumulations and fewer nodes to flush.
+// a warp's consecutive particles occupy few, densely filled cells: the scatter
+// then makes few reductions per particle.
 // ---------------------------------------------------------------------------
 // with_class: water particles before every other material (their keys offset
 // by S x MB), so that the non-water particles occupy the index range [Nl, N).
@@ -326,17 +324,6 @@ int sm_count() {
     cached[dev] = n;  // a plain int store: concurrent first calls write the same value
   }
   return cached[dev];
-}
-
-void max_shared_carveout(const void* kernel) {
-  static std::mutex lock;
-  static std::set<const void*> done;
-  std::lock_guard<std::mutex> g(lock);
-  if (done.count(kernel)) return;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           cudaSharedmemCarveoutMaxShared) != cudaSuccess)
-    cudaGetLastError();
-  done.insert(kernel);
 }
 
 void launch_iota(int* a, int N, cudaStream_t s) {

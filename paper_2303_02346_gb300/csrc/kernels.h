@@ -45,10 +45,6 @@ struct Tuning {
   int scatter_ctas = 3;       // resident 256-thread CTAs per SM of the fused step and G2P adjoint (3 or 4)
 };
 
-// Carve the SM's unified L1 / shared memory out at its largest shared part
-// for `kernel` (once per kernel): the 4-CTA builds of the scatter kernels need it.
-void max_shared_carveout(const void* kernel);
-
 // forward step stages
 // reset_count (nullable): an active-block counter to zero for the next step
 void launch_p2g(const Params& P, const Tuning& tu, const float* st_in, const uint32_t* tag, GridBuffers g,

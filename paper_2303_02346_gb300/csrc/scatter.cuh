@@ -1,29 +1,35 @@
-// Particle-to-grid scatter through a cell-binned shared-memory tile.
+// Particle-to-grid scatter, one warp at a time.
 //
-// A CTA owns a contiguous range of particles that the block sort keeps
-// spatially compact. It reduces the bounding box of their stencil origins
-// ("cells"). If the box plus the 3-node stencil fits in the tile and every
-// particle belongs to one scene:
-//   1. each thread writes its particle's record (fractional position f and the
-//      coefficients of its per-node contribution) into shared memory, counting-
-//      sorted by cell;
-//   2. work item (cell, o_x, o_y) over the occupied cells accumulates the
-//      contributions of all particles of that cell to its 3 nodes (o_z = 0..2)
-//      in registers, then adds them to the tile with one shared atomic per node
-//      and value;
-//   3. the CTA flushes every touched node with one global float4 reduction.
-// Particles of one cell hit the same 27 nodes, so step 2 replaces one atomic
-// per particle and node by one per cell and node; the 9 items of one cell sit
-// in neighbouring lanes, read the same records (shared-memory broadcast) and add
-// to distinct nodes. Otherwise (a range straddling scenes or spread too far)
-// each particle reduces straight into global memory.
+// The particle sort keeps the particles of a cell (stencil origin) together, so
+// the 32 particles of a warp lie in a few cells. A warp
+//   1. writes each particle's record (fractional position f and the
+//      coefficients of its per-node contribution) to its own shared memory;
+//   2. finds the particles of equal cell (match_any over the stencil origin's
+//      node index);
+//   3. takes three cells at a time, each with 9 lanes (a, b) = column of the
+//      stencil: a lane sums the contributions of the cell's particles to its
+//      column's three nodes in registers, reading the records as broadcasts,
+//      and adds the four values of each node with one global vector reduction.
+// No step needs another warp: there is no barrier, no zeroing and no size limit,
+// and the work of one warp overlaps the load latency of the others. A particle
+// of a warp that spans cells of any distance (or scenes) takes the same path.
+//
+// What bounds it: the instruction issue and load latency of the kernels around
+// it; the reductions (18 sectors per cell and warp) keep L2 below a fifth of
+// its rate. It replaced a shared-memory tile per CTA (cells binned and scanned
+// by the CTA, one shared FP32 atomic per cell, node and value, a flush, nine
+// barriers). Per launch on the 2M-particle dam break: fused step 237 -> 148 us
+// (215 at the tile's best launch shape), G2P adjoint 234 -> 147 (213), P2G
+// 190 -> 113; on the 200k-particle scene 35.6 -> 24.9, 33.5 -> 23.3 and
+// 30.9 -> 19.9. One cell at a time with a lane per node measured 160 and 154
+// us in place of 148 and 147: each lane then repeats the column's weights.
 //
 // The contribution of a particle with coefficients (c, M) to node x_i at
 // offset dpos = x_i - x_p = (o - f) dx (o = the node's offset in the stencil,
 // f = the particle's fractional position) is  W * (c + M dpos)  per value;
 // P2G's first value (mass) has no dpos term. The record stores the same
 // affine map in the node offset o: c + M dpos = c' + M' o with M' = M dx and
-// c' = c - M' f, so that step 2 needs no per-particle offset arithmetic.
+// c' = c - M' f, so that step 3 needs no per-particle offset arithmetic.
 #pragma once
 
 #include <climits>
@@ -32,194 +38,18 @@
 
 namespace mpm {
 
-constexpr int kTileCap = 1280;          // nodes (and cells) per tile (static shared memory <= 48 KB)
-constexpr int kRecF4 = 5;               // float4 per particle record
-// Resident threads per SM the G2P adjoint kernel is compiled for (3 CTAs of
-// 256 or 6 of 128: at most 85 registers a thread, and 3 x 47 KB of shared
-// memory; left to itself the compiler takes 118 registers and 2 CTAs), and,
-// as a launch choice for the fused step and the G2P adjoint, 4 CTAs of 256
-// at 64 registers, which needs the SM's shared memory carved out at its
-// maximum (4 x 47 KB).
+constexpr int kRecF4 = 5;  // float4 per particle record: 4 used, the fifth keeps 16-byte stores free of bank conflicts
+// Resident threads per SM the scatter kernels are compiled for: 3 CTAs of 256
+// or 6 of 128 (at most 85 registers a thread) and, as a launch choice for the
+// fused step and the G2P adjoint, 4 CTAs of 256 or 8 of 128 (64 registers).
 constexpr int kScatterResidentThreads = 768;
 constexpr int kScatterResidentThreadsHigh = 1024;
 
-// record (5 x float4): (f.x, f.y, w_z0, w_z1) (c_m, c'0, c'1, c'2) then the columns
-// of M' with a zero in front, (0, M'_0j, M'_1j, M'_2j) for j = 0, 1, 2;
-// value v (vector part) = c'_v + M'_v . o; P2G adds a mass value c_m.
 // NT = threads per CTA = particles per CTA (one each)
-// 128-byte aligned: the node accumulators double as the landing area of a
-// tensor-copy (TMA) of grid values before the scatter uses them.
 template <int NT>
-struct alignas(128) ScatterTile {
-  float acc[4][kTileCap];
-  int cnt[kTileCap];
+struct alignas(16) ScatterSmem {
   float4 rec[NT * kRecF4];
-  int occ[NT];  // occupied cells
-  int red[2][4][NT / 32];
-  int box[11];  // ox oy oz ex ey ez scene mode ncell nvalid nocc
-  float inv[4];  // 1 / ez, 1 / (ey ez), 1 / cz, 1 / (cy cz) for div_small
 };
-
-// q = a / d for 0 <= a < 2^20 and 0 < d < 2^10 from a float reciprocal of d
-// (inv = 1/d rounded): the float quotient is within 1 of the exact one, and
-// the remainder test corrects it. Replaces the integer division sequence
-// where tile indices are decoded.
-__device__ inline int div_small(int a, int d, float inv) {
-  int q = __float2int_rz(__int2float_rn(a) * inv);
-  const int r = a - q * d;
-  q += int(r >= d) - int(r < 0);
-  return q;
-}
-
-// Block-wide bounding box of the stencil origins and tile decision. Every
-// thread of the CTA must call it. On return the tile accumulators and cell
-// counts are zero when the tile is used.
-template <int NT>
-__device__ inline void scatter_setup(ScatterTile<NT>& T, bool valid, const int* base, int scene) {
-  const int nvalid = __syncthreads_count(valid);
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int vmin[4], vmax[4];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    vmin[d] = valid ? base[d] : INT_MAX;
-    vmax[d] = valid ? base[d] : INT_MIN;
-  }
-  vmin[3] = valid ? scene : INT_MAX;
-  vmax[3] = valid ? scene : INT_MIN;
-#pragma unroll
-  for (int d = 0; d < 4; ++d) {
-    int mn = __reduce_min_sync(0xffffffffu, vmin[d]);
-    int mx = __reduce_max_sync(0xffffffffu, vmax[d]);
-    if (lane == 0) {
-      T.red[0][d][wid] = mn;
-      T.red[1][d][wid] = mx;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int nw = blockDim.x >> 5;
-    int mn[4], mx[4];
-    for (int d = 0; d < 4; ++d) {
-      mn[d] = INT_MAX;
-      mx[d] = INT_MIN;
-      for (int w = 0; w < nw; ++w) {
-        mn[d] = min(mn[d], T.red[0][d][w]);
-        mx[d] = max(mx[d], T.red[1][d][w]);
-      }
-    }
-    bool any = mn[3] != INT_MAX;
-    long long cx = any ? (long long)mx[0] - mn[0] + 1 : 0, cy = any ? (long long)mx[1] - mn[1] + 1 : 0,
-              cz = any ? (long long)mx[2] - mn[2] + 1 : 0;
-    long long nodes = (cx + 2) * (cy + 2) * (cz + 2);
-    T.box[0] = mn[0];
-    T.box[1] = mn[1];
-    T.box[2] = mn[2];
-    T.box[3] = int(cx + 2);
-    T.box[4] = int(cy + 2);
-    T.box[5] = int(cz + 2);
-    T.box[6] = mn[3];
-    T.box[7] = (any && mn[3] == mx[3] && nodes <= kTileCap) ? 1 : 0;
-    T.box[8] = int(cx * cy * cz);
-    T.box[9] = nvalid;
-    T.box[10] = 0;
-    T.inv[0] = __frcp_rn(float(cz + 2));
-    T.inv[1] = __frcp_rn(float((cy + 2) * (cz + 2)));
-    T.inv[2] = __frcp_rn(float(cz > 0 ? cz : 1));
-    T.inv[3] = __frcp_rn(float(cy * cz > 0 ? cy * cz : 1));
-  }
-  __syncthreads();
-  if (T.box[7]) {
-    int nt = T.box[3] * T.box[4] * T.box[5];
-    for (int t = threadIdx.x; t < nt; t += blockDim.x) {
-      T.acc[0][t] = 0.0f;
-      T.acc[1][t] = 0.0f;
-      T.acc[2][t] = 0.0f;
-      T.acc[3][t] = 0.0f;
-    }
-    for (int t = threadIdx.x; t < T.box[8]; t += blockDim.x) T.cnt[t] = 0;
-  }
-  __syncthreads();
-}
-
-template <int NT>
-__device__ inline int cell_of(const ScatterTile<NT>& T, const int* base) {
-  int cy = T.box[4] - 2, cz = T.box[5] - 2;
-  return ((base[0] - T.box[0]) * cy + (base[1] - T.box[1])) * cz + (base[2] - T.box[2]);
-}
-
-// Exclusive scan of the cell counts in place (every thread must call it).
-template <int NT>
-__device__ inline void scan_cells(ScatterTile<NT>& T) {
-  __shared__ int wsum[NT / 32];
-  const int n = T.box[8];
-  const int per = (n + blockDim.x - 1) / blockDim.x;
-  const int lo = threadIdx.x * per;
-  int s = 0;
-  for (int i = 0; i < per; ++i)
-    if (lo + i < n) s += T.cnt[lo + i];
-  int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int x = s;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) wsum[wid] = x;
-  __syncthreads();
-  int pre = x - s;
-  for (int w = 0; w < wid; ++w) pre += wsum[w];
-  for (int i = 0; i < per; ++i)
-    if (lo + i < n) {
-      int c = T.cnt[lo + i];
-      T.cnt[lo + i] = pre;
-      pre += c;
-      if (c > 0) T.occ[atomicAdd(&T.box[10], 1)] = lo + i;
-    }
-  __syncthreads();
-}
-
-// Phase 1 (tile mode): place this particle's record, sorted by cell.
-// rank = the value returned by atomicAdd on the cell count.
-template <int NT>
-__device__ inline int scatter_count(ScatterTile<NT>& T, bool valid, const int* base) {
-  if (!valid) return -1;
-  return atomicAdd(&T.cnt[cell_of(T, base)], 1);
-}
-template <int NT>
-__device__ inline float4* scatter_slot(ScatterTile<NT>& T, const int* base, int rank) {
-  return T.rec + (T.cnt[cell_of(T, base)] + rank) * kRecF4;
-}
-
-// Phase 1 (tile mode): write the record of a particle with stencil sc
-// (fractional position f, weights w), mass value c_m and per-value
-// coefficients (c, M) (M row-major, 3 x 3) at its cell-sorted slot. The values
-// are laid out as two pairs, (mass, v0) and (v1, v2), each in one half of a
-// float4, so that step 2 accumulates them with packed two-lane FP32
-// instructions; the mass has no offset term (zero M' entries). The z weights
-// of offsets 0 and 1 replace f_z (the third is 1 minus their sum).
-// scatter_record_affine takes the coefficients already in the node-offset
-// form (c', M').
-template <int NT>
-__device__ inline void scatter_record_affine(ScatterTile<NT>& T, int rank, const Stencil& sc, float cm,
-                                             const float* cp, const float* Md) {
-  float4* r = scatter_slot(T, sc.base, rank);
-  r[0] = make_float4(sc.f[0], sc.f[1], sc.w[2][0], sc.w[2][1]);
-  r[1] = make_float4(cm, cp[0], cp[1], cp[2]);
-  r[2] = make_float4(0.0f, Md[0], Md[3], Md[6]);
-  r[3] = make_float4(0.0f, Md[1], Md[4], Md[7]);
-  r[4] = make_float4(0.0f, Md[2], Md[5], Md[8]);
-}
-template <int NT>
-__device__ inline void scatter_record(ScatterTile<NT>& T, int rank, const Stencil& sc, float cm,
-                                      const float* c, const float* M, float dx) {
-  const float* f = sc.f;
-  float Md[9], cp[3];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) Md[k] = M[k] * dx;
-#pragma unroll
-  for (int v = 0; v < 3; ++v) cp[v] = c[v] - (Md[3 * v] * f[0] + Md[3 * v + 1] * f[1] + Md[3 * v + 2] * f[2]);
-  scatter_record_affine(T, rank, sc, cm, cp, Md);
-}
 
 // Quadratic B-spline weight of stencil offset o as a polynomial in the
 // fractional position f in [0.5, 1.5): w_o(f) = k0 + k1 f + k2 f^2, from
@@ -230,77 +60,6 @@ __device__ inline void spline_poly(int o, float& k0, float& k1, float& k2) {
   k2 = o == 1 ? -1.0f : 0.5f;
 }
 
-// Phase 2 (tile mode, every thread must call it): per (occupied cell, o_x,
-// o_y) item, accumulate the cell's particles into its 3 nodes (o_z = 0, 1, 2)
-// in registers and add them to the tile. kMass: 4 values (mass first), else
-// the 3 vector values (the record's mass slot is zero and is not added).
-// The values travel as the pairs (mass, v0) and (v1, v2) through packed
-// two-lane FP32 fused multiply-adds and adds (per lane the same rounding as
-// the scalar fmaf and add).
-template <bool kMass, int NT>
-__device__ inline void scatter_accumulate(ScatterTile<NT>& T) {
-  const int ncell = T.box[8], nocc = T.box[10];
-  const int cy = T.box[4] - 2, cz = T.box[5] - 2;
-  const int ey = T.box[4], ez = T.box[5];
-  for (int item = threadIdx.x; item < 9 * nocc; item += blockDim.x) {
-    const int oc = item / 9, sub = item - 9 * oc;
-    const int oa = sub / 3, ob = sub - 3 * oa;
-    const int c = T.occ[oc];
-    const int start = T.cnt[c];
-    const int end = (c + 1 < ncell) ? T.cnt[c + 1] : T.box[9];
-    float ka0, ka1, ka2, kb0, kb1, kb2;
-    spline_poly(oa, ka0, ka1, ka2);
-    spline_poly(ob, kb0, kb1, kb2);
-    const float2 k0 = make_float2(ka0, kb0), k1 = make_float2(ka1, kb1), k2 = make_float2(ka2, kb2);
-    const float2 fa = make_float2(float(oa), float(oa)), fb = make_float2(float(ob), float(ob));
-    float2 acc[3][2];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) acc[q][0] = acc[q][1] = make_float2(0.0f, 0.0f);
-    for (int s = start; s < end; ++s) {
-      const float4* r = T.rec + s * kRecF4;
-      const float4 r0 = r[0], r1 = r[1], m0 = r[2], m1 = r[3], m2 = r[4];
-      const float2 fxy = make_float2(r0.x, r0.y);
-      const float2 wab = __ffma2_rn(__ffma2_rn(k2, fxy, k1), fxy, k0);  // (w_x(o_a), w_y(o_b))
-      const float wxy = wab.x * wab.y;
-      const float2 W01 = __fmul2_rn(make_float2(wxy, wxy), make_float2(r0.z, r0.w));
-      const float W[3] = {W01.x, W01.y, wxy - W01.x - W01.y};
-      // value pairs at o_z = 0, stepped by the third column of M' per unit o_z
-      float2 val[2] = {__ffma2_rn(make_float2(m1.x, m1.y), fb,
-                                  __ffma2_rn(make_float2(m0.x, m0.y), fa, make_float2(r1.x, r1.y))),
-                       __ffma2_rn(make_float2(m1.z, m1.w), fb,
-                                  __ffma2_rn(make_float2(m0.z, m0.w), fa, make_float2(r1.z, r1.w)))};
-      const float2 st[2] = {make_float2(m2.x, m2.y), make_float2(m2.z, m2.w)};
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const float2 w = make_float2(W[q], W[q]);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          acc[q][h] = __ffma2_rn(w, val[h], acc[q][h]);
-          if (q < 2) val[h] = __fadd2_rn(val[h], st[h]);
-        }
-      }
-    }
-    const int ci = div_small(c, cy * cz, T.inv[3]);
-    const int cjk = c - ci * (cy * cz);
-    const int cj = div_small(cjk, cz, T.inv[2]);
-    const int ck = cjk - cj * cz;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const int t = ((ci + oa) * ey + (cj + ob)) * ez + (ck + q);
-      if (kMass) {
-        atomicAdd(&T.acc[0][t], acc[q][0].x);
-        atomicAdd(&T.acc[1][t], acc[q][0].y);
-        atomicAdd(&T.acc[2][t], acc[q][1].x);
-        atomicAdd(&T.acc[3][t], acc[q][1].y);
-      } else {
-        atomicAdd(&T.acc[0][t], acc[q][0].y);
-        atomicAdd(&T.acc[1][t], acc[q][1].x);
-        atomicAdd(&T.acc[2][t], acc[q][1].y);
-      }
-    }
-  }
-}
-
 // Activate grid block b: the first caller to set its flag appends it to the
 // active-block list (the grid update clears the flag again).
 __device__ inline void activate_block(int* __restrict__ flags, int* __restrict__ list,
@@ -308,46 +67,7 @@ __device__ inline void activate_block(int* __restrict__ flags, int* __restrict__
   if (flags[b] == 0 && atomicExch(&flags[b], 1) == 0) list[atomicAdd(count, 1)] = int(b);
 }
 
-// Flush the tile to global memory (every thread must call it). If `flags` is
-// given, activates the grid blocks the tile covers.
-template <int NT>
-__device__ inline void scatter_flush(ScatterTile<NT>& T, float4* __restrict__ grid, const Params& P,
-                                     int* __restrict__ flags, int* __restrict__ list,
-                                     int* __restrict__ count) {
-  __syncthreads();
-  if (!T.box[7]) return;
-  const int ox = T.box[0], oy = T.box[1], oz = T.box[2];
-  const int ex = T.box[3], ey = T.box[4], ez = T.box[5], sc = T.box[6];
-  const int nt = ex * ey * ez;
-  for (int t = threadIdx.x; t < nt; t += blockDim.x) {
-    float a = T.acc[0][t], b = T.acc[1][t], c = T.acc[2][t], d = T.acc[3][t];
-    if (a != 0.0f || b != 0.0f || c != 0.0f || d != 0.0f) {
-      const int ti = div_small(t, ey * ez, T.inv[1]);
-      const int tjk = t - ti * (ey * ez);
-      const int tj = div_small(tjk, ez, T.inv[0]);
-      red_add_v4(grid + node_index(P, sc, ox + ti, oy + tj, oz + tjk - tj * ez), a, b, c, d);
-    }
-  }
-  if (flags) {
-    int bx0 = ox / kBlockEdge, by0 = oy / kBlockEdge, bz0 = oz / kBlockEdge;
-    int nbx = (ox + ex - 1) / kBlockEdge - bx0 + 1;
-    int nby = (oy + ey - 1) / kBlockEdge - by0 + 1;
-    int nbz = (oz + ez - 1) / kBlockEdge - bz0 + 1;
-    int nbt = nbx * nby * nbz;
-    if (threadIdx.x < nbt) {
-      const float inv_yz = __frcp_rn(float(nby * nbz)), inv_z = __frcp_rn(float(nbz));
-      for (int t = threadIdx.x; t < nbt; t += blockDim.x) {
-        const int tx = div_small(t, nby * nbz, inv_yz);
-        const int tyz = t - tx * (nby * nbz);
-        const int ty = div_small(tyz, nbz, inv_z);
-        const int bx = bx0 + tx, by = by0 + ty, bz = bz0 + tyz - ty * nbz;
-        activate_block(flags, list, count, (long long)sc * P.NB + (bx * P.nb + by) * P.nb + bz);
-      }
-    }
-  }
-}
-
-// Activate the blocks of one particle's stencil (used when the tile is off).
+// Activate the blocks of one cell's stencil.
 __device__ inline void mark_stencil_blocks(const Params& P, int scene, const int* base,
                                            int* __restrict__ flags, int* __restrict__ list,
                                            int* __restrict__ count) {
@@ -361,6 +81,131 @@ __device__ inline void mark_stencil_blocks(const Params& P, int scene, const int
     for (int by = b0[1]; by <= b1[1]; ++by)
       for (int bz = b0[2]; bz <= b1[2]; ++bz)
         activate_block(flags, list, count, (long long)scene * P.NB + (bx * P.nb + by) * P.nb + bz);
+}
+
+// Activate the grid blocks that the stencils of a warp's cells touch (every
+// lane must call it; leaders: the lanes that hold one cell each). If the cells
+// share a scene and the blocks around them form a box of at most 12, one lane
+// marks each block of the box, so that a single load tests them all; a warp
+// spread wider marks cell by cell. (One lane per cell walking its up to 8
+// blocks put as many dependent loads in a row.)
+__device__ inline void mark_warp_blocks(const Params& P, unsigned leaders, bool leader, int scene, const int* base,
+                                        int* __restrict__ flags, int* __restrict__ list, int* __restrict__ count) {
+  constexpr unsigned kAll = 0xffffffffu;
+  if (leaders == 0u) return;
+  int lo[3], nb[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    lo[d] = __reduce_min_sync(kAll, leader ? base[d] : INT_MAX) / kBlockEdge;
+    nb[d] = (__reduce_max_sync(kAll, leader ? base[d] : 0) + 2) / kBlockEdge - lo[d] + 1;
+  }
+  const int smin = __reduce_min_sync(kAll, leader ? scene : INT_MAX);
+  const int smax = __reduce_max_sync(kAll, leader ? scene : 0);
+  // each factor is at least 1 and at most 256
+  const int yz = nb[1] * nb[2], total = nb[0] * yz;
+  if (smin == smax && total <= 12) {
+    const int lane = threadIdx.x & 31;
+    if (lane < total) {
+      const int tx = lane / yz, r = lane - tx * yz, ty = r / nb[2];
+      activate_block(flags, list, count, (long long)smin * P.NB +
+                                             ((lo[0] + tx) * P.nb + lo[1] + ty) * P.nb + lo[2] + r - ty * nb[2]);
+    }
+  } else if (leader) {
+    mark_stencil_blocks(P, scene, base, flags, list, count);
+  }
+}
+
+// Scatter of the warp's particles (every lane must call it). rec: the warp's
+// 32 records. valid: this lane holds a particle with stencil sc in `scene`, mass
+// value cm (kMass) and coefficients c' (cp) and M' (Md, row-major 3 x 3) in
+// node-offset form. The values travel as v0 (with the mass beside it) and the
+// pair (v1, v2) through packed two-lane FP32 fused multiply-adds (per lane the
+// rounding of the scalar fmaf). flags (nullable): activates the grid blocks
+// the stencils touch.
+template <bool kMass>
+__device__ inline void warp_scatter(float4* rec, const Params& P, bool valid, int scene, const Stencil& sc, float cm,
+                                    const float* cp, const float* Md, float4* __restrict__ grid,
+                                    int* __restrict__ flags, int* __restrict__ list, int* __restrict__ count) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  // node index of the stencil origin (all scenes' nodes number fewer than 2^31)
+  const int key = valid ? int(node_index(P, scene, sc.base[0], sc.base[1], sc.base[2])) : -1;
+  if (valid) {
+    float4* r = rec + lane * kRecF4;
+    r[0] = make_float4(sc.f[0], sc.f[1], sc.f[2], cm);
+    r[1] = make_float4(cp[0], Md[0], Md[1], Md[2]);
+    r[2] = make_float4(cp[1], cp[2], Md[3], Md[6]);
+    r[3] = make_float4(Md[4], Md[7], Md[5], Md[8]);
+  }
+  const unsigned peers = __match_any_sync(kAll, key);
+  const bool leader = valid && (peers & ((1u << lane) - 1u)) == 0u;
+  unsigned leaders = __ballot_sync(kAll, leader);
+  __syncwarp();  // the records are written
+  if (flags) mark_warp_blocks(P, leaders, leader, scene, sc.base, flags, list, count);
+  // this lane's column (a, b) of the stencil and the column's weight polynomials
+  const int sub = lane / 9, col = lane - 9 * sub;
+  const int oa = col / 3, ob = col - 3 * oa;
+  float ka0, ka1, ka2, kb0, kb1, kb2;
+  spline_poly(oa, ka0, ka1, ka2);
+  spline_poly(ob, kb0, kb1, kb2);
+  const float2 k0 = make_float2(ka0, kb0), k1 = make_float2(ka1, kb1), k2 = make_float2(ka2, kb2);
+  const float fa = float(oa), fb = float(ob);
+  const float2 fa2 = make_float2(fa, fa), fb2 = make_float2(fb, fb);
+  const int off = (oa * P.n + ob) * P.n;
+  while (leaders) {
+    // the next three cells, one per group of 9 lanes
+    const unsigned rest1 = leaders & (leaders - 1u), rest2 = rest1 & (rest1 - 1u);
+    const unsigned mine = sub == 0 ? leaders : sub == 1 ? rest1 : sub == 2 ? rest2 : 0u;
+    const int l = mine ? __ffs(mine) - 1 : lane;
+    unsigned m = __shfl_sync(kAll, peers, l);
+    const int node = __shfl_sync(kAll, key, l);
+    leaders = rest2 & (rest2 - 1u);
+    if (!mine) m = 0u;
+    float2 s01[3], s23[3];  // (mass, v0), (v1, v2) at the column's nodes c = 0, 1, 2
+#pragma unroll
+    for (int c = 0; c < 3; ++c) s01[c] = s23[c] = make_float2(0.0f, 0.0f);
+    while (m) {
+      const float4* r = rec + (__ffs(m) - 1) * kRecF4;
+      m &= m - 1u;
+      const float4 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3];
+      const float2 fxy = make_float2(r0.x, r0.y), fz = make_float2(r0.z, r0.z);
+      const float2 wab = __ffma2_rn(__ffma2_rn(k2, fxy, k1), fxy, k0);  // (w_x(a), w_y(b))
+      const float wxy = wab.x * wab.y;
+      // z weights of offsets 0 and 1; the third is 1 minus their sum
+      const float2 wz = __ffma2_rn(__ffma2_rn(make_float2(0.5f, -1.0f), fz, make_float2(-1.5f, 2.0f)), fz,
+                                   make_float2(1.125f, -0.25f));
+      const float2 W01 = __fmul2_rn(make_float2(wxy, wxy), wz);
+      const float W[3] = {W01.x, W01.y, wxy - W01.x - W01.y};
+      // values at c = 0, stepped by the third column of M' per node
+      float v0 = fmaf(r1.z, fb, fmaf(r1.y, fa, r1.x));
+      float2 v12 = __ffma2_rn(make_float2(r3.x, r3.y), fb2,
+                              __ffma2_rn(make_float2(r2.z, r2.w), fa2, make_float2(r2.x, r2.y)));
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float2 w2 = make_float2(W[c], W[c]);
+        if (kMass)
+          s01[c] = __ffma2_rn(w2, make_float2(r0.w, v0), s01[c]);
+        else
+          s01[c].y = fmaf(W[c], v0, s01[c].y);
+        s23[c] = __ffma2_rn(w2, v12, s23[c]);
+        if (c < 2) {
+          v0 += r1.w;
+          v12 = __fadd2_rn(v12, make_float2(r3.z, r3.w));
+        }
+      }
+    }
+    if (mine) {
+      float4* g = grid + node + off;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if (kMass)
+          red_add_v4(g + c, s01[c].x, s01[c].y, s23[c].x, s23[c].y);
+        else
+          red_add_v4(g + c, s01[c].y, s23[c].x, s23[c].y, 0.0f);
+      }
+    }
+    __syncwarp();
+  }
 }
 
 }  // namespace mpm
