@@ -317,11 +317,13 @@ long long sim_kernel_launches(sim_h h);
  * steps between two re-sorts run as one persistent launch (0, 1; on devices
  * with cooperative launches and without rigid materials), whether the fused
  * G2P stages each CTA's box of grid velocities in shared memory with one
- * tensor-copy (TMA) load (0, 1), how many 256-thread CTAs of the fused step
- * and the G2P adjoint each SM holds (3 at 80 registers, 4 at 64) and, without
- * checkpoints, the re-sort period (4, 8, 16, 32 steps). Each candidate runs n_steps steps (0 = 10; at most
- * max_steps when checkpointing or a tool is on), plus the reverse sweep in
- * gradient mode, with CUDA events around the kernels it affects. The choice
+ * tensor-copy (TMA) load (0, 1), how many threads of the fused step and the
+ * G2P adjoint each SM holds, in 256s (3 at 80 registers, 4 at 64) and, without
+ * checkpoints, the re-sort period (4, 8, 16, 32 steps). A handle that is not
+ * tuned takes these shapes from rules on its particle count. Each candidate
+ * runs n_steps steps (0 = 10; at most max_steps when checkpointing or a tool
+ * is on), plus the reverse sweep in gradient mode, with CUDA events around the
+ * kernels it affects. The choice
  * is cached per (GPU, particle count, scenes, grid, checkpoint interval) for
  * the process. The trajectory is restarted from the initial state (pending
  * loss gradients are not allowed). choices (nullable, 8 ints) receives the

@@ -17,6 +17,12 @@
 namespace mpm {
 
 constexpr int fX = 0, fV = 3, fC = 6, fF = 15;
+// Resident threads per SM the P2G adjoint is compiled for (6 CTAs of 128, 80
+// registers; the spills fall in the solids' SVD adjoint): 124 us on the
+// 2M-particle dam break against 131 at 128 registers with the SVD held across
+// the gather, 126 at 96 registers. The kExt build keeps 128 registers (its
+// viscous branch alone spills 300 bytes at 80).
+constexpr int kGatherResidentThreads = 768;
 static inline int blocks_for(long long n, int t) { return int((n + t - 1) / t); }
 
 // Adjoint of G2P of step n for one particle (the gather part). Inputs: the
@@ -124,7 +130,7 @@ __device__ inline void g2p_adj_scatter(ScatterSmem<NT>& T, const Params& P, bool
                       nullptr, nullptr);
 }
 
-// kHigh: 4 resident CTAs of 256 per SM (64 registers) instead of 3
+// kHigh: 1024 resident threads per SM (64 registers) instead of 768
 template <int NT, bool kHigh = false>
 __global__ void __launch_bounds__(NT, (kHigh ? kScatterResidentThreadsHigh : kScatterResidentThreads) / NT)
 g2p_adj_kernel(Params P, const float* __restrict__ st_n, const float* __restrict__ st_n1,
@@ -300,6 +306,14 @@ __device__ __noinline__ float viscous_liquid_adjoint(const MatParams& M, const f
   return sFG * a / (3.0f * J);
 }
 
+// A load the compiler neither merges with an earlier one of the same address
+// nor moves across one.
+__device__ __forceinline__ float load_again(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+
 // Adjoint of P2G of step n (with the constitutive adjoint) for one particle.
 // Inputs: the state of step n (st_n), C^{n+1} (st_n1), the stored SVD of the
 // trial F^n, the partial adjoint of x^n and the adjoint F' of F^{n+1} in adj,
@@ -319,7 +333,7 @@ __device__ inline void p2g_adj_particle(const Params& P, int p, const MatParams&
 #pragma unroll
   for (int d = 0; d < 3; ++d) prefetch_l2(adj + (fX + d) * N + p);
   prefetch_l2(adj + fF * N + p);
-  float x[3], v[3], C[9], tau[9], U[9], sg[3], V[9];
+  float x[3], v[3], C[9], tau[9];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     x[d] = st_n[(fX + d) * N + p];
@@ -340,11 +354,9 @@ __device__ inline void p2g_adj_particle(const Params& P, int p, const MatParams&
     for (int k = 0; k < 9; ++k) tau[k] = (k % 4 == 0) ? pr : 0.0f;
   } else {
     // SVD of the trial F stored by the recompute of this step
+    float U[9], sg[3];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      U[k] = svd_n[sslot(P, k, p)];
-      V[k] = svd_n[sslot(P, 12 + k, p)];
-    }
+    for (int k = 0; k < 9; ++k) U[k] = svd_n[sslot(P, k, p)];
 #pragma unroll
     for (int k = 0; k < 3; ++k) sg[k] = svd_n[sslot(P, 9 + k, p)];
     solid_tau_from_svd<kExt>(M, U, sg, tau);
@@ -454,7 +466,21 @@ __device__ inline void p2g_adj_particle(const Params& P, int p, const MatParams&
   float Cv[9];  // C^n's adjoint through a viscous liquid's trial F
 #pragma unroll
   for (int k = 0; k < 9; ++k) Cv[k] = 0.0f;
+  // the SVD again (and a viscous liquid's C): read a second time instead of
+  // being held in 21 registers across the node gather
+  float U[9], sg[3], V[9];
+  if (!rigid && (!liquid || viscous)) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      U[k] = load_again(svd_n + sslot(P, k, p));
+      V[k] = load_again(svd_n + sslot(P, 12 + k, p));
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) sg[k] = load_again(svd_n + sslot(P, 9 + k, p));
+  }
   if (viscous) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) C[k] = load_again(st_n + (fC + k) * N + p);
     Fb[0] = adj[fF * N + p] * det3(G) + viscous_liquid_adjoint(M, U, sg, V, taub, C, P.dt, J, Cv);
   } else if (liquid) {
     Fb[0] = adj[fF * N + p] * det3(G) + M.lam * (2.0f * J - 1.0f) * (taub[0] + taub[4] + taub[8]);
@@ -475,8 +501,8 @@ __device__ inline void p2g_adj_particle(const Params& P, int p, const MatParams&
   for (int k = 0; k < 9; ++k) Cb[k] = m * Ab[k] + Cv[k];
 }
 
-template <bool kExt>
-__global__ void __launch_bounds__(512)
+template <int NT, bool kExt>
+__global__ void __launch_bounds__(NT, kExt ? 512 / NT : kGatherResidentThreads / NT)
 p2g_adj_kernel(Params P, const float* __restrict__ st_n, const float* __restrict__ st_n1,
                const uint32_t* __restrict__ tag, const float* __restrict__ svd_n,
                float* __restrict__ adj, const float4* __restrict__ gadj_m) {
@@ -504,9 +530,9 @@ p2g_adj_kernel(Params P, const float* __restrict__ st_n, const float* __restrict
 // Adjoint of P2G of step n fused with the adjoint of G2P of step n - 1: the
 // adjoint of the state of step n stays in registers; only the partial adjoint
 // of x^{n-1} and the adjoint of F^n are written back. Compiled for two CTAs
-// of 256 (three of 128) per SM: at most 128 (170) registers a thread.
-template <int NT, bool kExt>
-__global__ void __launch_bounds__(NT, NT >= 256 ? 2 : 3)
+// of 256 per SM, or three (kMore: four) of 128: at most 128, 168 (128) registers.
+template <int NT, bool kExt, bool kMore = false>
+__global__ void __launch_bounds__(NT, NT >= 256 ? 2 : (kMore ? 4 : 3))
 adj_fused_kernel(Params P, const float* __restrict__ st_prev, const float* __restrict__ st_n,
                  const float* __restrict__ st_n1, const uint32_t* __restrict__ tag,
                  const float* __restrict__ svd_n, const float* __restrict__ Fp_prev,
@@ -602,8 +628,14 @@ void launch_adj_fused(const Params& P, const Tuning& tu, const float* st_prev, c
                       float* adj, const float4* gadj_m, const float4* gv_prev, float4* gadj_v,
                       cudaStream_t s) {
   if (P.N == 0) return;
-  auto k = tu.scatter_threads == 128 ? (P.ext ? adj_fused_kernel<128, true> : adj_fused_kernel<128, false>)
-                                     : (P.ext ? adj_fused_kernel<256, true> : adj_fused_kernel<256, false>);
+  // 3 CTAs of 128 per SM at 168 registers or 4 at 128, by their waves: sweeps
+  // of 0.53 / 0.56 ms (8k particles), 0.70 / 0.73 (100k), 1.96 / 1.85 (200k), 4.57
+  // / 4.19 (500k)
+  const bool more = tight_build_wins(blocks_for(P.N, 128), sm_count(), 3, 4);
+  auto k = tu.scatter_threads == 128
+               ? (more ? (P.ext ? adj_fused_kernel<128, true, true> : adj_fused_kernel<128, false, true>)
+                       : (P.ext ? adj_fused_kernel<128, true> : adj_fused_kernel<128, false>))
+               : (P.ext ? adj_fused_kernel<256, true> : adj_fused_kernel<256, false>);
   const int nt = tu.scatter_threads == 128 ? 128 : 256;
   k<<<blocks_for(P.N, nt), nt, 0, s>>>(P, st_prev, st_n, st_n1, tag, svd_n, Fp_prev, adj, gadj_m, gv_prev, gadj_v);
 }
@@ -613,7 +645,9 @@ void launch_p2g_adj(const Params& P, const Tuning& tu, const float* st_n, const 
                     cudaStream_t s) {
   if (P.N == 0) return;
   const int t = tu.gather_threads;
-  auto k = P.ext ? p2g_adj_kernel<true> : p2g_adj_kernel<false>;
+  auto k = t == 128   ? (P.ext ? p2g_adj_kernel<128, true> : p2g_adj_kernel<128, false>)
+           : t == 256 ? (P.ext ? p2g_adj_kernel<256, true> : p2g_adj_kernel<256, false>)
+                      : (P.ext ? p2g_adj_kernel<512, true> : p2g_adj_kernel<512, false>);
   k<<<blocks_for(P.N, t), t, 0, s>>>(P, st_n, st_n1, tag, svd_n, adj, gadj_m);
 }
 

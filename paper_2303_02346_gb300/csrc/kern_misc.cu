@@ -326,6 +326,28 @@ int sm_count() {
   return cached[dev];
 }
 
+// Measured (GB300, gradient runs, us per launch unless stated):
+// * CTAs of 128 against 256: fused step 148 / 150 (2M particles), 24.9 / 25.5
+//   (200k), 17.4 / 18.2 (100k), 11.6 / 12.1 (8k); P2G adjoint 124 / 126 and
+//   G2P 82 / 98 (2M). 64 a CTA: no faster at any size down to 8k.
+// * fused step and G2P adjoint at 8 resident CTAs (64 registers) against 6
+//   (80): 148 / 160 and 147 / 162 (2M), 45 / 47 and 46 / 50 (500k), 19.0 / 21.9
+//   and 17.7 / 22.1 (130k: one wave against two); 25.3 / 24.9 and 23.8 / 23.3
+//   (200k: two waves either way), 18.1 / 17.4 (100k: one wave either way).
+// * one adjoint kernel against two, whole reverse sweep: 0.53 / 0.74 ms (8k
+//   particles), 0.70 / 0.74 (100k), 1.86 / 1.90 (200k), 4.22 / 4.42 (500k), 7.85
+//   / 7.86 (1M), 15.1 / 14.7 (2M), 11.8 / 11.5 (3.2M in 64 scenes): fused saves a
+//   launch and the adjoint state's round trip, but its 128 registers leave half
+//   the warps, which counts once the chip is full for many waves.
+constexpr int kFuseBelow = 1000000;
+Tuning default_tuning(int N) {
+  Tuning tu;
+  const long long ctas = blocks_for(N, tu.scatter_threads);
+  tu.scatter_ctas = tight_build_wins(ctas, sm_count(), 768 / tu.scatter_threads, 1024 / tu.scatter_threads) ? 4 : 3;
+  tu.fuse_adjoint = N < kFuseBelow ? 1 : 0;
+  return tu;
+}
+
 void launch_iota(int* a, int N, cudaStream_t s) {
   if (N == 0) return;
   iota_kernel<<<blocks_for(N, 256), 256, 0, s>>>(a, N);

@@ -34,16 +34,28 @@ struct GridBuffers {
   int ovf_bit = 0;
 };
 
-// Launch shapes chosen by the autotuner (sim_autotune).
+// Launch shapes: default_tuning's rules, or the autotuner's choice (sim_autotune).
 struct Tuning {
-  int scatter_threads = 256;  // p2g / g2p_adj: 128 or 256 particles per CTA
-  int gather_threads = 256;   // g2p / p2g_adj: 128, 256 or 512 threads per CTA
+  int scatter_threads = 128;  // p2g / g2p2g / g2p_adj / adj_fused: 128 or 256 particles per CTA
+  int gather_threads = 128;   // g2p / p2g_adj: 128, 256 or 512 threads per CTA
   int grid_blocks = 4;        // grid_update / grid_adj: 1, 2 or 4 grid blocks (64 threads each) per CTA
   int fuse_adjoint = 0;       // 1: P2G adjoint of step n fused with the G2P adjoint of step n - 1
   int persistent = 0;         // 1: forward runs between re-sorts as one persistent cooperative launch
   int stage_gather = 0;       // 1: fused G2P stages each CTA's grid box in shared memory by a TMA load
-  int scatter_ctas = 3;       // resident 256-thread CTAs per SM of the fused step and G2P adjoint (3 or 4)
+  int scatter_ctas = 3;       // resident threads per SM of the fused step and G2P adjoint, in 256s (3 or 4)
 };
+
+// Whether the build of a kernel that keeps `tight` CTAs resident per SM (fewer
+// registers a thread, some spills) needs fewer waves for `ctas` CTAs than the
+// one that keeps `wide`. Where both need as many waves the wide build is the
+// faster one, elsewhere the tight one.
+inline bool tight_build_wins(long long ctas, int sms, int wide, int tight) {
+  const long long w = (long long)sms * wide, t = (long long)sms * tight;
+  return (ctas + t - 1) / t < (ctas + w - 1) / w;
+}
+
+// Default launch shapes for N particles on the current device.
+Tuning default_tuning(int N);
 
 // forward step stages
 // reset_count (nullable): an active-block counter to zero for the next step

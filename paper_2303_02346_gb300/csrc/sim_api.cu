@@ -56,7 +56,7 @@ struct mpm_sim {
   sim_config cfg;
   std::vector<int> counts, offsets;
   Params P;
-  Tuning tu;  // launch shapes (sim_autotune)
+  Tuning tu;  // launch shapes (default_tuning, sim_autotune)
   cudaStream_t stream = nullptr;
   int N = 0, S = 0, n = 0;
   long long n3tot = 0, nflags = 0;
@@ -977,6 +977,7 @@ sim_status sim_create(const sim_config* c, sim_h* out) {
   h->offsets[0] = 0;
   for (int s = 0; s < h->S; ++s) h->offsets[s + 1] = h->offsets[s] + h->counts[s];
   h->N = int(Ntot);
+  h->tu = default_tuning(h->N);
   h->n = c->grid_n;
   h->stream = static_cast<cudaStream_t>(c->cuda_stream);
   h->k = c->checkpoint_every;
@@ -1810,18 +1811,16 @@ sim_status sim_autotune(sim_h h, int n_steps, int* choices) {
     if (t < best) best = t, pick = c;
   }
   h->tu.scatter_threads = pick;
-  if (h->tu.scatter_threads == 256) {
-    // resident CTAs of the fused step and the G2P adjoint: 3 (80 registers)
-    // or 4 (64 registers, some spills)
-    best = 1e30;
-    pick = h->tu.scatter_ctas;
-    for (int c : {3, 4}) {
-      h->tu.scatter_ctas = c;
-      double t = trial({"p2g", "g2p2g", "g2p_adj", "adj_fused"});
-      if (t < best) best = t, pick = c;
-    }
-    h->tu.scatter_ctas = pick;
+  // resident threads per SM of the fused step and the G2P adjoint: 768 (80
+  // registers) or 1024 (64 registers, some spills)
+  best = 1e30;
+  pick = h->tu.scatter_ctas;
+  for (int c : {3, 4}) {
+    h->tu.scatter_ctas = c;
+    double t = trial({"p2g", "g2p2g", "g2p_adj", "adj_fused"});
+    if (t < best) best = t, pick = c;
   }
+  h->tu.scatter_ctas = pick;
   best = 1e30;
   pick = h->tu.gather_threads;
   for (int c : ga_c) {
