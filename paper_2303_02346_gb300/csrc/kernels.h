@@ -99,13 +99,18 @@ cudaError_t launch_barrier_selftest(unsigned* bar, int blocks, unsigned expected
 struct SortBuffers {
   uint32_t* key;   // N
   uint32_t* rank;  // N
-  uint32_t* bins;  // 2 n_bins + 1 (the particle sort keys water and the other materials apart)
+  uint32_t* bins;  // 2 n_bins (the particle sort keys water and the other materials apart): a cell's
+                   // count, then its first slot; zero outside a sort
+  uint32_t* blk_cnt;    // 2 n_bins / 64: particles per 4^3 block; zero outside a sort
+  uint32_t* blk_start;  // the block's first slot (of blocks that hold particles)
   uint32_t* tile_sums;
   int n_bins;      // scenes x Morton codes per scene
 };
 // Sort by (class: water first, scene, Morton code of the stencil-origin cell)
 void launch_sort(const Params& P, const float* st_in, const uint32_t* tag_in, const int* pid_in,
                  float* st_out, uint32_t* tag_out, int* pid_out, SortBuffers sb, cudaStream_t s);
+// Zero the bins and block counts that launch_bin (share.h) left for its readers
+void launch_bin_clear(const Params& P, SortBuffers sb, cudaStream_t s);
 // water particles among the tags into *out (device int)
 void launch_count_water(const Params& P, const uint32_t* tag, int* out, cudaStream_t s);
 

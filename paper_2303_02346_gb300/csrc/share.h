@@ -13,9 +13,11 @@ namespace mpm {
 
 // Cell bins of the particles at their current positions, without moving
 // them: key[p] = (scene, Morton code of the stencil-origin cell), rank[p] =
-// position of p among the particles of its key, bins = exclusive prefix of
-// the key counts (start of each key; a key's end is the next key's start,
-// or N for the last key). Uses the sort buffers.
+// position of p among the particles of its key, bins = first slot of each
+// key of the 4^3 blocks that hold particles (64 consecutive keys, blk_cnt
+// nonzero; a key ends at the next one's first slot, a block's last key at
+// blk_start + blk_cnt). Uses the sort buffers; launch_bin_clear (kernels.h)
+// must follow the last kernel that reads them.
 void launch_bin(const Params& P, const float* st, const uint32_t* tag, SortBuffers sb, cudaStream_t s);
 
 // Neighbour arrays in bin order. pk[slot] = (x, c) with c = exp(-ell[q] /

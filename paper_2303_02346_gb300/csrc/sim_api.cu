@@ -377,7 +377,7 @@ void do_sort(sim_h h, const float* st_in, const uint32_t* tag_in, const int* pid
              uint32_t* tag_out, int* pid_out, cudaStream_t s) {
   Prof pr(h, "sort", s);
   launch_sort(h->P, st_in, tag_in, pid_in, st_out, tag_out, pid_out, h->sb, s);
-  h->launches += h->P.N > 0 ? 5 : 3;
+  h->launches += h->P.N > 0 ? 6 : 0;
 }
 
 // Wait for the stream and read the error word. The word is copied to pinned
@@ -1013,8 +1013,9 @@ sim_status sim_create(const sim_config* c, sim_h* out) {
             dalloc(h, &h->rows, (size_t)N * kStateFields) && dalloc(h, &h->inv, N) &&
             cudaMallocHost(&h->words, 3 * sizeof(int)) == cudaSuccess;
   h->sb.n_bins = int(nbins);
-  ok = ok && dalloc(h, &h->sb.key, N) && dalloc(h, &h->sb.rank, N) && dalloc(h, &h->sb.bins, 2 * nbins + 1) &&
-       dalloc(h, &h->sb.tile_sums, 2 * nbins / 4096 + 2);
+  ok = ok && dalloc(h, &h->sb.key, N) && dalloc(h, &h->sb.rank, N) && dalloc(h, &h->sb.bins, 2 * nbins) &&
+       dalloc(h, &h->sb.blk_cnt, nbins / 32) && dalloc(h, &h->sb.blk_start, nbins / 32) &&
+       dalloc(h, &h->sb.tile_sums, nbins / 32 / 4096 + 2);
   if (ok && h->P.tool) {
     h->n_act_max = (h->max_steps + h->spa - 1) / h->spa;
     ok = dalloc(h, &h->pose0, (size_t)7 * h->S) && dalloc(h, &h->actions, (size_t)h->S * h->n_act_max * 6) &&
@@ -1048,7 +1049,9 @@ sim_status sim_create(const sim_config* c, sim_h* out) {
     sim_destroy(h);
     return SIM_E_OOM;
   }
-  // zero-initialised invariants: acc, flags, gadj_v; X0 = rest state at the origin
+  // zero-initialised invariants: acc, flags, sort bins, gadj_v; X0 = rest state at the origin
+  cudaMemsetAsync(h->sb.bins, 0, sizeof(uint32_t) * 2 * (size_t)nbins, h->stream);
+  cudaMemsetAsync(h->sb.blk_cnt, 0, sizeof(uint32_t) * (size_t)(nbins / 32), h->stream);
   cudaMemsetAsync(h->acc, 0, sizeof(float4) * h->n3tot, h->stream);
   cudaMemsetAsync(h->gv, 0, sizeof(float4) * h->n3tot, h->stream);
   cudaMemsetAsync(h->flags, 0, sizeof(int) * h->nflags, h->stream);
@@ -1457,7 +1460,7 @@ static sim_status nbr_prepare(sim_h h, const char* where, int scene, const float
   if (e != cudaSuccess) return cuda_fail(h, e, where);
   launch_bin(h->P, h->W, h->tag_cur, h->sb, h->stream);
   launch_nbr_pack(h->P, h->W, h->pid_cur, h->sb, s_ell, g ? s_g : nullptr, *lo, *cnt, tau, h->nb, h->stream);
-  h->launches += N > 0 ? 6 : 3;
+  h->launches += N > 0 ? 5 : 0;
   return SIM_OK;
 }
 
@@ -1474,10 +1477,14 @@ sim_status sim_attraction_loss(sim_h h, int scene, const float* ell, float radiu
   {
     Prof pr(h, "attraction");
     float* seed = seed_buffer(h, h->step);
-    if (!seed) return fail(h, SIM_E_OOM, "sim_attraction_loss: out of device memory");
+    if (!seed) {
+      launch_bin_clear(h->P, h->sb, h->stream);
+      return fail(h, SIM_E_OOM, "sim_attraction_loss: out of device memory");
+    }
     launch_attraction(h->P, h->tag_cur, h->sb, h->nb, radius, weight, seed, h->dloss, h->stream);
+    launch_bin_clear(h->P, h->sb, h->stream);
   }
-  h->launches += h->N > 0 ? 1 : 0;
+  h->launches += h->N > 0 ? 2 : 0;
   cudaError_t e = cudaMemcpyAsync(loss_out, h->dloss, sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "sim_attraction_loss");
   return check_err(h, "sim_attraction_loss");
@@ -1494,8 +1501,9 @@ sim_status sim_share_gradients(sim_h h, int scene, const float* ell, float radiu
   {
     Prof pr(h, "share");
     launch_share(h->P, h->tag_cur, h->pid_cur, h->sb, h->nb, radius, lo, s_out, h->stream);
+    launch_bin_clear(h->P, h->sb, h->stream);
   }
-  h->launches += h->N > 0 ? 1 : 0;
+  h->launches += h->N > 0 ? 2 : 0;
   cudaError_t e = to_caller(h, out, s_out, sizeof(float) * 3 * cnt, on_device);
   if (e != cudaSuccess) return cuda_fail(h, e, "sim_share_gradients");
   return check_err(h, "sim_share_gradients");
