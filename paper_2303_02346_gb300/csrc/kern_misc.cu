@@ -278,21 +278,25 @@ __global__ void inverse_perm_kernel(const int* __restrict__ pid, int* __restrict
 }
 
 // dst[f][p'] = src[f][inv_from[pid_to[p']]]: writes coalesced, reads gathered
-// (the two orders differ by one re-sort, so the reads stay mostly local)
+// (the two orders differ by one re-sort, so the reads stay mostly local). Both
+// orders have the same first n_first particles, of which only the first
+// f_first fields are copied (water carries J alone of F's nine).
 __global__ void permute_state_kernel(const float* __restrict__ src, float* __restrict__ dst,
                                      const int* __restrict__ inv_from, const int* __restrict__ pid_to, int N,
-                                     int fields) {
+                                     int n_first, int f_first, int fields) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= N) return;
   const long long p = inv_from[pid_to[q]];
-  for (int f = 0; f < fields; ++f) dst[(long long)f * N + q] = src[(long long)f * N + p];
+  const int nf = q < n_first ? f_first : fields;
+#pragma unroll 8
+  for (int f = 0; f < nf; ++f) dst[(long long)f * N + q] = src[(long long)f * N + p];
 }
 
 void launch_permute_state(const float* src, float* dst, const int* pid_from, const int* pid_to, int* inv, int N,
-                          int fields, cudaStream_t s) {
+                          int n_first, int f_first, int fields, cudaStream_t s) {
   if (N == 0) return;
   inverse_perm_kernel<<<blocks_for(N, 256), 256, 0, s>>>(pid_from, inv, N);
-  permute_state_kernel<<<blocks_for(N, 256), 256, 0, s>>>(src, dst, inv, pid_to, N, fields);
+  permute_state_kernel<<<blocks_for(N, 256), 256, 0, s>>>(src, dst, inv, pid_to, N, n_first, f_first, fields);
 }
 
 void launch_gather_rows(const float* src, float* dst, const int* pid, int N, int fields,

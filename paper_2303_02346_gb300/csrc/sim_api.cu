@@ -247,6 +247,7 @@ int* ck_pids(sim_h h, int c) { return h->ck_pid + (size_t)c * h->N; }
 // buffer's last slot; with rigid materials (whose recompute rereads F) every
 // state keeps 24.
 constexpr int kChunkFields = 16;
+constexpr int fF = 15;  // first field of F
 float* chunk_state(sim_h h, int b, int j, int L) {
   if (h->rigid) return h->chunk[b] + (size_t)(j - 1) * state_floats(h);
   const size_t slot = (size_t)kChunkFields * h->N;
@@ -366,10 +367,10 @@ void stage_rigid(sim_h h, float* st, const uint32_t* tag, const int* pid, float*
   launch_rigid_project(h->P, st, tag, pid, h->rb, rec, s);
   h->launches += h->N > 0 ? 3 : 0;
 }
-void stage_rigid_adj(sim_h h, const uint32_t* tag, const int* pid, const float* rec, cudaStream_t s) {
+void stage_rigid_adj(sim_h h, float* adj, const uint32_t* tag, const int* pid, const float* rec, cudaStream_t s) {
   if (!h->rigid) return;
   Prof pr(h, "rigid_adj", s);
-  launch_rigid_adjoint(h->P, h->adj, tag, pid, h->rb, rec, s);
+  launch_rigid_adjoint(h->P, adj, tag, pid, h->rb, rec, s);
   h->launches += h->N > 0 ? 3 : 0;
 }
 
@@ -468,7 +469,6 @@ void restart(sim_h h) {
   h->need_sort = true;
   clear_seeds(h);
   h->rec_from = -1;
-  if (h->adj) cudaMemsetAsync(h->adj, 0, state_floats(h) * sizeof(float), h->stream);
   cudaMemsetAsync(h->err, 0, sizeof(int), h->stream);
 }
 
@@ -896,7 +896,7 @@ sim_status loss_site(sim_h h, const char* where, int step, LossSite* out) {
 void finish_loss_site(sim_h h, const LossSite& s) {
   if (s.ckpt < 0 || h->N == 0) return;
   float* tmp = h->rows + (size_t)3 * h->N;
-  launch_permute_state(h->rows, tmp, ck_pids(h, s.ckpt), ck_pids(h, s.ckpt - 1), h->inv, h->N, 3, h->stream);
+  launch_permute_state(h->rows, tmp, ck_pids(h, s.ckpt), ck_pids(h, s.ckpt - 1), h->inv, h->N, 0, 3, 3, h->stream);
   launch_add_fields(s.seed, tmp, (long long)3 * h->N, 0, h->stream);
   h->launches += 3;
 }
@@ -1064,7 +1064,6 @@ sim_status sim_create(const sim_config* c, sim_h* out) {
   if (N) cudaMemcpy(h->tag0, tags.data(), sizeof(uint32_t) * N, cudaMemcpyHostToDevice);
   if (h->k > 0) {
     cudaMemsetAsync(h->gadj_v, 0, sizeof(float4) * h->n3tot, h->stream);
-    cudaMemsetAsync(h->adj, 0, NS * sizeof(float), h->stream);
   }
   if (h->P.tool) {
     std::vector<float> p0(7 * h->S, 0.0f);
@@ -1516,9 +1515,10 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
   const int T = h->step, K = h->k, N = h->N;
   const Params& P = h->P;
   // Device work of the reverse sweep on stream s (forks to rstream for the
-  // overlapped recompute and joins back): ends with the adjoint of the initial
-  // state in caller order in `rows`, the action gradients in `action_grad`,
-  // and the adjoint state cleared.
+  // overlapped recompute and joins back): starts from a zero adjoint state in
+  // `adj`, which changes between `adj` and `rows` at every chunk boundary, and
+  // ends with the adjoint of the initial state (checkpoint 0's order) in one
+  // of them, the action gradients in `action_grad`.
   const bool overlap = h->nbuf >= 2 && !h->prof;
   // the forward that reached max_steps left its last chunks [rec_from, nch)
   // in the buffers their sweeps read (rec_from = nch: every chunk is recomputed)
@@ -1530,10 +1530,12 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
   // steps whose loss seeds the sweep adds into the adjoint state (and clears)
   const std::vector<int> seeded(h->seeded.begin(), h->seeded.end());
   auto has_seed = [&](int t) { return h->seeded.count(t) > 0; };
+  float* A = h->adj;       // the adjoint state
+  float* spare = h->rows;  // its other buffer
   auto inject = [&](int t, cudaStream_t st) {
     if (!has_seed(t)) return;
     Prof pr(h, "seed", st);
-    launch_add_fields(h->adj, h->seed_buf[t], (long long)kSeedFields * N, 1, st);
+    launch_add_fields(A, h->seed_buf[t], (long long)kSeedFields * N, 1, st);
     h->launches += N > 0 ? 1 : 0;
   };
   auto enqueue = [&](cudaStream_t s_in) {
@@ -1546,6 +1548,9 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
       cudaStreamWaitEvent(h->hstream, h->ev_start, 0);
       s = h->hstream;
     }
+    A = h->adj;
+    spare = h->rows;
+    cudaMemsetAsync(A, 0, state_floats(h) * sizeof(float), s);
     if (h->P.tool) cudaMemsetAsync(h->tool_grad, 0, sizeof(float) * h->S * h->max_steps * kToolGradFields, s);
     const int nch = (T + K - 1) / K;
     auto recompute = [&](int c, int b, cudaStream_t rs) { recompute_chunk(h, c, b, T, rs); };
@@ -1584,7 +1589,7 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
       // runs the two adjoints unfused to make room for that.
       const int* pids = ck_pids(h, c);
       inject(s0 + L, s);
-      stage_rigid_adj(h, tag, pids, rig_step(h, b, L - 1), s);
+      stage_rigid_adj(h, A, tag, pids, rig_step(h, b, L - 1), s);
       // a compact buffer's grid of step j is expanded into gscr before the
       // G2P adjoint of step j + 1 reads it; it stays there for the grid
       // adjoint of step j
@@ -1592,7 +1597,7 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
       {
         GridBuffers g = step_grid(h, b, L - 1);
         Prof pr(h, "g2p_adj", s);
-        launch_g2p_adj(P, h->tu, state(L - 1), state(L), tag, g.Fp, h->adj, g.gv, h->gadj_v, s);
+        launch_g2p_adj(P, h->tu, state(L - 1), state(L), tag, g.Fp, A, g.gv, h->gadj_v, s);
         h->launches += N > 0 ? 1 : 0;
       }
       for (int j = L - 1; j >= 0; --j) {
@@ -1606,26 +1611,26 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
           GridBuffers gp = step_grid(h, b, j - 1);
           {
             Prof pr(h, "p2g_adj", s);
-            launch_p2g_adj(P, h->tu, state(j), state(j + 1), tag, g.svd, h->adj, h->gadj_m, s);
+            launch_p2g_adj(P, h->tu, state(j), state(j + 1), tag, g.svd, A, h->gadj_m, s);
           }
           inject(s0 + j, s);
-          stage_rigid_adj(h, tag, pids, rig_step(h, b, j - 1), s);
+          stage_rigid_adj(h, A, tag, pids, rig_step(h, b, j - 1), s);
           stage_expand(h, b, j - 1, s);
           {
             Prof pr(h, "g2p_adj", s);
-            launch_g2p_adj(P, h->tu, state(j - 1), state(j), tag, gp.Fp, h->adj, gp.gv, h->gadj_v, s);
+            launch_g2p_adj(P, h->tu, state(j - 1), state(j), tag, gp.Fp, A, gp.gv, h->gadj_v, s);
           }
           h->launches += N > 0 ? 2 : 0;
         } else if (j > 0) {
           GridBuffers gp = step_grid(h, b, j - 1);
           stage_expand(h, b, j - 1, s);
           Prof pr(h, "adj_fused", s);
-          launch_adj_fused(P, h->tu, state(j - 1), state(j), state(j + 1), tag, g.svd, gp.Fp, h->adj,
+          launch_adj_fused(P, h->tu, state(j - 1), state(j), state(j + 1), tag, g.svd, gp.Fp, A,
                            h->gadj_m, gp.gv, h->gadj_v, s);
           h->launches += N > 0 ? 1 : 0;
         } else {
           Prof pr(h, "p2g_adj", s);
-          launch_p2g_adj(P, h->tu, state(0), state(1), tag, g.svd, h->adj, h->gadj_m, s);
+          launch_p2g_adj(P, h->tu, state(0), state(1), tag, g.svd, A, h->gadj_m, s);
           h->launches += N > 0 ? 1 : 0;
         }
       }
@@ -1640,13 +1645,11 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
       if (c > 0) {
         // adjoint of the re-sort at step s0: order of checkpoint c -> order of chunk c - 1
         Prof pr(h, "permute", s);
-        launch_permute_state(h->adj, h->rows, ck_pids(h, c), ck_pids(h, c - 1), h->inv, N, kStateFields, s);
-        cudaMemcpyAsync(h->adj, h->rows, state_floats(h) * sizeof(float), cudaMemcpyDeviceToDevice, s);
+        launch_permute_state(A, spare, ck_pids(h, c), ck_pids(h, c - 1), h->inv, N, P.Nl, fF + 1, kStateFields, s);
+        std::swap(A, spare);
         h->launches += N > 0 ? 2 : 0;
       }
     }
-    launch_gather_rows(h->adj, h->rows, ck_pids(h, 0), N, kStateFields, N, 0, 1, s);
-    h->launches += N > 0 ? 1 : 0;
     if (h->P.tool) {
       cudaMemsetAsync(h->action_grad, 0, sizeof(float) * h->S * h->n_actions * 6, s);
       {
@@ -1656,7 +1659,6 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
       }
       h->launches += 1;
     }
-    cudaMemsetAsync(h->adj, 0, state_floats(h) * sizeof(float), s);
     if (overlap) {
       cudaEventRecord(h->ev_join, s);
       cudaStreamWaitEvent(s_in, h->ev_join, 0);
@@ -1693,18 +1695,23 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
   if (!done) enqueue(h->stream);
   h->rec_from = -1;  // the sweep's recomputes reuse the chunk buffers
   h->seeded.clear();   // the sweep added and cleared every pending seed
-  // outputs in caller order
-  sim_status st = check_err(h, "sim_backward");
-  if (st != SIM_OK) return st;
+  // outputs in caller order, straight into device buffers, through the spare
+  // buffer for host ones; one wait for all of it. The sweep left the adjoint in
+  // `adj` or `rows` by its number of chunk boundaries (a replayed graph did not
+  // run the swaps above).
+  A = (nch_all - 1) % 2 ? h->rows : h->adj;
+  spare = (nch_all - 1) % 2 ? h->adj : h->rows;
   cudaError_t e = cudaSuccess;
   if ((dLdx0 || dLdv0) && N > 0) {
-    // rows holds the initial state's adjoint in caller order, kStateFields
-    // floats per particle: x at 0..2, v at 3..5; one strided copy each
-    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    const size_t pitch = kStateFields * sizeof(float), w = 3 * sizeof(float);
-    if (dLdx0) e = cudaMemcpy2DAsync(dLdx0, w, h->rows, pitch, w, N, kind, h->stream);
-    if (e == cudaSuccess && dLdv0) e = cudaMemcpy2DAsync(dLdv0, w, h->rows + 3, pitch, w, N, kind, h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    float* host[2] = {dLdx0, dLdv0};
+    float* dev[2] = {dLdx0, dLdv0};
+    for (int q = 0; q < 2 && !on_device; ++q) dev[q] = host[q] ? spare + (size_t)3 * q * N : nullptr;
+    launch_read_state(P, A, h->tag0, ck_pids(h, 0), 0, N, dev[0], dev[1], nullptr, nullptr, h->stream);
+    h->launches += 1;
+    e = cudaGetLastError();
+    for (int q = 0; q < 2 && !on_device && e == cudaSuccess; ++q)
+      if (host[q])
+        e = cudaMemcpyAsync(host[q], dev[q], sizeof(float) * 3 * N, cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "sim_backward");
   }
   if (dLdactions && h->P.tool) {
