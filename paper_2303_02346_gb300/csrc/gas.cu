@@ -15,11 +15,14 @@
 // graphs and replayed.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "mpm_gas.h"
+#include "sur_ptx.cuh"
 
 namespace {
 
@@ -263,9 +266,68 @@ jacobi_kernel(Geo g, const float* __restrict__ p_in, float* __restrict__ p_out, 
 // cell). A CTA covers 128 cells along k times 8 rows along j.
 __device__ __forceinline__ float f4(const float4& v, int t) { return t == 0 ? v.x : t == 1 ? v.y : t == 2 ? v.z : v.w; }
 
+// 1 / (number of fluid neighbours) for every set of neighbour bits (0 for
+// none), in shared memory: the first 64 threads of a CTA fill it.
+__device__ __forceinline__ void fill_weights(float* tab, int tid) {
+  if (tid < 64) {
+    const int nf = __popc(tid);
+    tab[tid] = nf == 0 ? 0.0f : 1.0f / float(nf);
+  }
+}
+
+// The neighbour bits of a thread's 4 cells along k when none but the grid's own
+// ends along k are missing, and the weights of the first and the last cell then.
+struct Ends {
+  uint32_t bits;
+  float w0, w3;
+};
+__device__ __forceinline__ Ends ends_of(bool first_in_row, bool last_in_row) {
+  Ends e;
+  e.bits = 0x3f3f3f3fu & ~(first_in_row ? 32u : 0u) & ~(last_in_row ? 16u << 24 : 0u);
+  e.w0 = first_in_row ? 1.0f / 5.0f : 1.0f / 6.0f;
+  e.w3 = last_in_row ? 1.0f / 5.0f : 1.0f / 6.0f;
+  return e;
+}
+
+// Sweep of 4 cells along k: P their values, Q their neighbours at +i, -i, +j,
+// -j, pl and pr the cells before and after them (zeros for cells outside the
+// grid), R the right-hand side without its mean, M4 the neighbour bits (a byte a
+// cell), tab from fill_weights. p is zero on solid cells before and after every
+// sweep, so the sums need no tests; the bits matter only where a cell is solid
+// or misses a neighbour. A row's ends are told apart from other missing
+// neighbours because every warp holds one: testing each cell there made the
+// pair kernel's warps issue 438 instructions a plane, looking the weights up
+// 317, and with the ends set apart 291.
+__device__ __forceinline__ float4 sweep4(const float4& P, const float4 (&Q)[4], float pl, float pr, const float4& R,
+                                         uint32_t M4, const Ends& e, const float* tab, float h2) {
+  float w[4] = {e.w0, 1.0f / 6.0f, 1.0f / 6.0f, e.w3}, out[4];
+  const bool plain = M4 == e.bits;
+  if (!plain) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) w[t] = tab[(M4 >> (8 * t)) & 63u];
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const float zp = t < 3 ? f4(P, t + 1) : pr;
+    const float zm = t > 0 ? f4(P, t - 1) : pl;
+    const float s = f4(Q[0], t) + f4(Q[1], t) + f4(Q[2], t) + f4(Q[3], t) + zp + zm;
+    // every operation spelled out: all forms of the sweep round alike
+    out[t] = fmaf(1.0f - kOmega, f4(P, t), __fmul_rn(__fmul_rn(kOmega, fmaf(-h2, f4(R, t), s)), w[t]));
+  }
+  if (!plain) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (M4 & (uint32_t(kSolidBit) << (8 * t))) out[t] = 0.0f;
+  }
+  return make_float4(out[0], out[1], out[2], out[3]);
+}
+
 __global__ void __launch_bounds__(kThreads)
 jacobi4_kernel(Geo g, const float* __restrict__ p_in, float* __restrict__ p_out, const float* __restrict__ rhs,
                const uint8_t* __restrict__ nbr, const float* __restrict__ mean_p, int first) {
+  __shared__ float tab[64];
+  fill_weights(tab, threadIdx.y * kBx + threadIdx.x);
+  __syncthreads();
   const int n = g.n;
   const int k0 = (blockIdx.x * kBx + threadIdx.x) * 4;
   const int j = blockIdx.y * kBy + threadIdx.y;
@@ -273,61 +335,193 @@ jacobi4_kernel(Geo g, const float* __restrict__ p_in, float* __restrict__ p_out,
   if (k0 >= n || j >= n) return;
   const int n1 = n, n2 = n * n;
   const int c = (i * n + j) * n + k0;
-  float4 P = make_float4(0.f, 0.f, 0.f, 0.f), Q[4];
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 P = zero, Q[4] = {zero, zero, zero, zero};
   float pl = 0.0f, pr = 0.0f;
   if (!first) {
     P = *reinterpret_cast<const float4*>(p_in + c);
-    Q[0] = *reinterpret_cast<const float4*>(p_in + (i + 1 < n ? c + n2 : c));
-    Q[1] = *reinterpret_cast<const float4*>(p_in + (i > 0 ? c - n2 : c));
-    Q[2] = *reinterpret_cast<const float4*>(p_in + (j + 1 < n ? c + n1 : c));
-    Q[3] = *reinterpret_cast<const float4*>(p_in + (j > 0 ? c - n1 : c));
+    if (i + 1 < n) Q[0] = *reinterpret_cast<const float4*>(p_in + c + n2);
+    if (i > 0) Q[1] = *reinterpret_cast<const float4*>(p_in + c - n2);
+    if (j + 1 < n) Q[2] = *reinterpret_cast<const float4*>(p_in + c + n1);
+    if (j > 0) Q[3] = *reinterpret_cast<const float4*>(p_in + c - n1);
     pl = k0 > 0 ? p_in[c - 1] : 0.0f;
     pr = k0 + 4 < n ? p_in[c + 4] : 0.0f;
   }
-  const float4 R = *reinterpret_cast<const float4*>(rhs + c);
+  float4 R = *reinterpret_cast<const float4*>(rhs + c);
   const uint32_t M4 = *reinterpret_cast<const uint32_t*>(nbr + c);
   const float mean = mean_p ? *mean_p : 0.0f;
-  const float h2 = g.dx * g.dx;
-  float out[4];
-#pragma unroll
-  for (int t = 0; t < 4; ++t) {
-    const uint32_t m = (M4 >> (8 * t)) & 0xffu;
-    if (m & kSolidBit) {
-      out[t] = 0.0f;
-      continue;
-    }
-    float s = 0.0f, pc = 0.0f;
-    if (!first) {
-      const float zp = t < 3 ? f4(P, t + 1) : pr;
-      const float zm = t > 0 ? f4(P, t - 1) : pl;
-      s = ((m & 1) ? f4(Q[0], t) : 0.0f) + ((m & 2) ? f4(Q[1], t) : 0.0f) + ((m & 4) ? f4(Q[2], t) : 0.0f) +
-          ((m & 8) ? f4(Q[3], t) : 0.0f) + ((m & 16) ? zp : 0.0f) + ((m & 32) ? zm : 0.0f);
-      pc = f4(P, t);
-    }
-    const int nf = __popc(m & 63u);
-    const float inv_nf = nf == 0 ? 0.0f : nf == 1 ? 1.0f : nf == 2 ? 0.5f : nf == 3 ? (1.0f / 3.0f) : nf == 4 ? 0.25f
-                       : nf == 5 ? 0.2f : (1.0f / 6.0f);
-    out[t] = (1.0f - kOmega) * pc + kOmega * (s - h2 * (f4(R, t) - mean)) * inv_nf;
-  }
-  *reinterpret_cast<float4*>(p_out + c) = make_float4(out[0], out[1], out[2], out[3]);
+  R = make_float4(R.x - mean, R.y - mean, R.z - mean, R.w - mean);
+  *reinterpret_cast<float4*>(p_out + c) = sweep4(P, Q, pl, pr, R, M4, ends_of(k0 == 0, k0 + 4 == n), tab, g.dx * g.dx);
 }
 
-// un -= central-difference gradient of p (p mirrored across solid faces)
+// Two sweeps in one pass over memory. A sweep is bound by DRAM (13 bytes a
+// cell: p, right-hand side and bits read, p written), so the second one is
+// taken from registers and shared memory. A CTA owns a strip of R - 2 rows
+// along j (all of k, 4 cells a thread, R rows of threads) and marches along i
+// through `seg` planes. A strip's rows of a plane are consecutive in memory, so
+// one bulk copy brings p (R + 2 rows) and one the right-hand side into a ring of
+// kStages planes, up to three planes ahead (~100 KB in flight per SM; with
+// plain loads one plane ahead the pair was no faster). At plane i the CTA sweeps its R rows once (i +- 1 in registers, j +- 1
+// from the ring), writes the result to a second ring of three planes, and
+// after the step's one barrier sweeps the inner R - 2 rows of plane i - 1 a
+// second time. The rows and planes of the halo are swept by both neighbours
+// ((R / (R - 2)) x ((seg + 2) / seg) of the first sweep's work, none of the
+// second's). Values are those of two single sweeps. Every wait is bounded;
+// one that runs out sets *err. Measured per sweep (us, against one sweep a pass with
+// the same arithmetic; before it 5.4 / - / 20.6 / 40.1): 5.6 / 4.2 at 128^3, 8.9 /
+// 10.0 at 160^3, 13.4 / 17.0 at 192^3, 26.7 / 35.5 at 256^3: the pair is bound by
+// instruction issue (0.78 of the slots), the single sweep by DRAM, or by L2
+// where everything fits there.
+constexpr int kStages = 4;
+struct PairShape {
+  int tx, rows, strips, seg, grid_i;
+  size_t smem;
+};
+__host__ __device__ inline size_t pair_stage_f4(int tx, int rows) { return (size_t)(2 * rows + 2) * tx; }
+
+__global__ void __launch_bounds__(1024, 1)
+jacobi2_kernel(Geo g, const float* __restrict__ p_in, float* __restrict__ p_out, const float* __restrict__ rhs,
+               const uint8_t* __restrict__ nbr, const float* __restrict__ mean_p, int first, int seg,
+               int* __restrict__ err) {
+  extern __shared__ __align__(128) float4 sm[];
+  __shared__ uint64_t bar[kStages];
+  __shared__ float tab[64];
+  const int n = g.n, n2 = n * n;
+  const int tx = threadIdx.x, ty = threadIdx.y, TX = blockDim.x, R = blockDim.y;
+  const int tid = ty * TX + tx, lane = tid & 31;
+  const int plane = R * TX, per = (2 * R + 2) * TX;  // float4 of a swept plane and of a stage
+  const int j0 = blockIdx.x * (R - 2);               // first inner row
+  const int j = j0 + ty - 1;
+  const bool row = j >= 0 && j < n;
+  const bool inner = row && ty >= 1 && ty < R - 1;
+  const int i0 = blockIdx.y * seg, i1 = min(i0 + seg, n);
+  const int col = j * n + 4 * tx;  // only used for rows inside the grid
+  // the value one cell before / after a thread's 4 comes from the neighbouring
+  // lane when that holds the same row, else from shared memory (0 at the ends)
+  const bool sl = tx > 0 && lane > 0, sr = tx + 1 < TX && lane < 31;
+  const bool el = tx > 0 && lane == 0, er = tx + 1 < TX && lane == 31;
+  const Ends ends = ends_of(tx == 0, tx + 1 == TX);
+  const float mean = mean_p ? *mean_p : 0.0f, h2 = g.dx * g.dx;
+  const int last = i1 - i0 + 2;  // plane i0 - 1 + o has ordinal o, 0 <= o <= last
+  // sm: 3 planes of the first sweep, then kStages x (R + 2 rows of p, R rows of
+  // the right-hand side); all zero, which rows outside the grid (and p in the
+  // first sweep of all) stay
+  for (int q = tid; q < 3 * plane + kStages * per; q += plane) sm[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  fill_weights(tab, tid);
+  if (tid == 0) {
+    for (int q = 0; q < kStages; ++q) sur::mbar_init(bar + q, 1);
+    sur::fence_barrier_init();
+  }
+  sur::fence_proxy_async_smem();  // the zeros come before the copies
+  __syncthreads();
+  // thread 0: bring the plane of ordinal o into its slot (planes outside the
+  // grid complete their phase without data)
+  auto issue = [&](int o) {
+    uint64_t* b = bar + o % kStages;
+    const int i = i0 - 1 + o;
+    if (i < 0 || i >= n) {
+      sur::mbar_arrive(b);
+      return;
+    }
+    float4* sp = sm + 3 * plane + (o % kStages) * per;
+    float4* srh = sp + (R + 2) * TX;
+    const int pa = max(j0 - 2, 0), pb = min(j0 + R, n);      // rows [pa, pb) of p
+    const int ra = max(j0 - 1, 0), rb = min(j0 + R - 1, n);  // rows [ra, rb) of the right-hand side
+    const uint32_t pbytes = first ? 0u : uint32_t(pb - pa) * n * 4u, rbytes = uint32_t(rb - ra) * n * 4u;
+    sur::mbar_arrive_expect_tx(b, pbytes + rbytes);
+    if (!first) sur::bulk_g2s(sp + (pa - (j0 - 2)) * TX, p_in + (size_t)i * n2 + (size_t)pa * n, pbytes, b);
+    sur::bulk_g2s(srh + (ra - (j0 - 1)) * TX, rhs + (size_t)i * n2 + (size_t)ra * n, rbytes, b);
+  };
+  if (tid == 0)
+    for (int o = 0; o < kStages && o <= last; ++o) issue(o);
+  auto await = [&](int o) {
+    if (!sur::mbar_wait(bar + o % kStages, (o / kStages) & 1, nullptr)) atomicOr(err, 1);
+  };
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  // outside the grid the solid bits are set: the sweep gives 0
+  const uint8_t* nb = nbr + col;
+  auto load_m = [&](int i) -> uint32_t {
+    return row && i >= 0 && i < n ? __ldg(reinterpret_cast<const uint32_t*>(nb + i * n2)) : 0x40404040u;
+  };
+  float4* const mine = sm + tid;                                // this thread's place in swept plane 0
+  const float4* const mine_p = sm + 3 * plane + tid + TX;      // and in stage 0's p
+  const float4* const mine_r = sm + 3 * plane + tid + per - plane;  // and right-hand side
+  uint32_t m = load_m(i0 - 1), mn = load_m(i0), mp = 0x40404040u;
+  const float4 far = (row && !first && i0 >= 2) ? __ldg(reinterpret_cast<const float4*>(p_in + (i0 - 2) * n2 + col)) : zero;
+  await(0);
+  await(1);
+  float4 a0 = far, a1 = i0 > 0 ? mine_p[0] : zero;
+  float4 s0 = zero, s1 = zero, rp = zero;  // first sweep of planes i - 2 and i - 1, right-hand side of i - 1
+  int now = 0, before = 2;                 // swept plane of i and of i - 1 in the ring
+  float* out = p_out + (i0 - 2) * n2 + col;  // only used for planes and rows inside the grid
+  for (int o = 0; o < last; ++o) {
+    const int i = i0 - 1 + o;
+    const uint32_t mnn = load_m(i + 2);
+    const float4 a2 = i + 1 < n ? mine_p[((o + 1) % kStages) * per] : zero;
+    const float4* sp = mine_p + (o % kStages) * per;
+    float4 r = mine_r[(o % kStages) * per];
+    r = make_float4(r.x - mean, r.y - mean, r.z - mean, r.w - mean);
+    float4 s2;
+    {
+      const float4 Q[4] = {a2, a0, sp[TX], sp[-TX]};
+      float pl = __shfl_up_sync(0xffffffffu, a1.w, 1), pr = __shfl_down_sync(0xffffffffu, a1.x, 1);
+      pl = sl ? pl : 0.0f;
+      pr = sr ? pr : 0.0f;
+      if (el) pl = sp[-1].w;
+      if (er) pr = sp[1].x;
+      s2 = sweep4(a1, Q, pl, pr, r, m, ends, tab, h2);
+    }
+    mine[now * plane] = s2;
+    if (tid < 32 && o + 2 <= last) await(o + 2);  // read by every warp after the barrier
+    __syncthreads();
+    if (tid == 0 && o + kStages <= last) issue(o + kStages);  // plane i's slot is not read again
+    {
+      // second sweep of plane i - 1 (rows outside the strip compute it unused)
+      const float4* c = mine + before * plane;
+      const float4 Q[4] = {s2, s0, ty < R - 1 ? c[TX] : zero, ty > 0 ? c[-TX] : zero};
+      float pl = __shfl_up_sync(0xffffffffu, s1.w, 1), pr = __shfl_down_sync(0xffffffffu, s1.x, 1);
+      pl = sl ? pl : 0.0f;
+      pr = sr ? pr : 0.0f;
+      if (el) pl = c[-1].w;
+      if (er) pr = c[1].x;
+      const float4 w = sweep4(s1, Q, pl, pr, rp, mp, ends, tab, h2);
+      if (inner && o >= 2) *reinterpret_cast<float4*>(out) = w;
+    }
+    out += n2;
+    s0 = s1;
+    s1 = s2;
+    a0 = a1;
+    a1 = a2;
+    rp = r;
+    mp = m;
+    m = mn;
+    mn = mnn;
+    before = now;
+    now = now == 2 ? 0 : now + 1;
+  }
+}
+
+// out = un - central-difference gradient of p (p mirrored across solid faces),
+// 0 on solid cells: the projected velocity, straight into the new state
 __global__ void __launch_bounds__(kThreads)
-gradient_kernel(Geo g, const float* __restrict__ p, const uint8_t* __restrict__ nbr, float* __restrict__ un) {
+gradient_kernel(Geo g, const float* __restrict__ p, const uint8_t* __restrict__ nbr, const float* __restrict__ un,
+                float* __restrict__ out) {
   int i, j, k;
   long long c;
   if (!my_cell(g.n, i, j, k, c)) return;
   const uint8_t m = nbr[c];
-  if (m & kSolidBit) return;
   const long long n1 = g.n, n2 = (long long)g.n * g.n, n3 = g.n3;
+  if (m & kSolidBit) {
+    out[c] = out[n3 + c] = out[2 * n3 + c] = 0.0f;
+    return;
+  }
   const float pc = p[c];
   const long long st[3] = {n2, n1, 1};
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const float pp = (m & (1 << (2 * a))) ? p[c + st[a]] : pc;
     const float pm = (m & (2 << (2 * a))) ? p[c - st[a]] : pc;
-    un[a * n3 + c] -= (pp - pm) * g.inv2dx;
+    out[a * n3 + c] = un[a * n3 + c] - (pp - pm) * g.inv2dx;
   }
 }
 
@@ -363,7 +557,8 @@ gradient_t_kernel(Geo g, const float* __restrict__ v, const uint8_t* __restrict_
 }
 
 // ubar = v - D^T (m - mean) on fluid cells, 0 on solid cells (the advection's
-// solid mask); m = the swept adjoint, *mean_p its mean over the fluid cells.
+// solid mask); m = the swept adjoint, *mean_p its mean over the fluid cells. The
+// density's adjoint (fourth field) is not projected and only passes the mask.
 __global__ void __launch_bounds__(kThreads)
 divergence_t_kernel(Geo g, const float* __restrict__ v, const float* __restrict__ mm, const uint8_t* __restrict__ nbr,
                     const float* __restrict__ mean_p, float* __restrict__ ubar) {
@@ -373,9 +568,10 @@ divergence_t_kernel(Geo g, const float* __restrict__ v, const float* __restrict_
   const long long n1 = g.n, n2 = (long long)g.n * g.n, n3 = g.n3;
   const uint8_t m = nbr[c];
   if (m & kSolidBit) {
-    ubar[c] = ubar[n3 + c] = ubar[2 * n3 + c] = 0.0f;
+    ubar[c] = ubar[n3 + c] = ubar[2 * n3 + c] = ubar[3 * n3 + c] = 0.0f;
     return;
   }
+  ubar[3 * n3 + c] = v[3 * n3 + c];
   const float mean = *mean_p;
   const long long st[3] = {n2, n1, 1};
 #pragma unroll
@@ -389,39 +585,61 @@ divergence_t_kernel(Geo g, const float* __restrict__ v, const float* __restrict_
 }
 
 // Transposed advection: scatter (ubar_adv, dbar_adv) of every fluid cell onto
-// the trilinear corners (one vector atomic per corner) and add the
-// back-trace's derivative to the cell's own velocity adjoint. acc (float4
-// per cell) is zero on entry and receives the adjoint of the packed fields
-// (buoyancy-updated velocity, density).
+// the trilinear corners and add the back-trace's derivative to the cell's own
+// velocity adjoint. acc (float4 per cell) is zero on entry and receives the
+// adjoint of the packed fields (buoyancy-updated velocity, density).
+// Bound by the vector atomics: neighbouring cells along k (the lanes of a warp)
+// mostly trace back to neighbouring corners, so where a lane's far corners in k
+// are the next lane's near ones it hands them over and they are added together
+// (5 atomics a cell instead of 9).
 __global__ void __launch_bounds__(kThreads)
 advect_t_kernel(Geo g, const float4* __restrict__ pk, const uint8_t* __restrict__ nbr,
                 const float* __restrict__ ubar, const float* __restrict__ dbar, float4* __restrict__ acc) {
+  constexpr unsigned kAll = 0xffffffffu;
   int i, j, k;
   long long c;
-  if (!my_cell(g.n, i, j, k, c)) return;
-  if (nbr[c] & kSolidBit) return;
+  bool act = my_cell(g.n, i, j, k, c);
+  act = act && !(nbr[c] & kSolidBit);
   const long long n3 = g.n3;
-  const float4 ub = pk[c];
+  float4 A = make_float4(0.f, 0.f, 0.f, 0.f), ub = A;
+  if (act) {
+    A = make_float4(ubar[c], ubar[n3 + c], ubar[2 * n3 + c], dbar[c]);
+    ub = pk[c];
+  }
+  act = act && (A.x != 0.0f || A.y != 0.0f || A.z != 0.0f || A.w != 0.0f);
+  if (!__any_sync(kAll, act)) return;
   const float X[3] = {i - g.dt_dx * ub.x, j - g.dt_dx * ub.y, k - g.dt_dx * ub.z};
   const Tri T = tri_of(X, g.n);
-  const float4 A = make_float4(ubar[c], ubar[n3 + c], ubar[2 * n3 + c], dbar[c]);
-  const bool any = A.x != 0.0f || A.y != 0.0f || A.z != 0.0f || A.w != 0.0f;
-  if (!any) return;
+  // near corner of this cell's stencil (-2: no contribution, links to nothing)
+  const long long q0 = act ? cid(g.n, T.i0[0], T.i0[1], T.i0[2]) : -2;
+  const long long qn = __shfl_down_sync(kAll, q0, 1);
+  // the next lane's near corners are this lane's far ones: same row, next cell
+  const bool give = act && (threadIdx.x & 31) < 31 && qn == q0 + 1 && T.i0[2] + 1 < g.n;
+  const bool take = __shfl_up_sync(kAll, int(give), 1) && (threadIdx.x & 31) > 0;
   float gX[3] = {0.f, 0.f, 0.f};
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int b = 0; b < 2; ++b)
+    for (int b = 0; b < 2; ++b) {
+      const float w0 = corner_w(T, a, b, 0), w1 = corner_w(T, a, b, 1);
+      float4 near = make_float4(w0 * A.x, w0 * A.y, w0 * A.z, w0 * A.w);
+      const float4 far = make_float4(w1 * A.x, w1 * A.y, w1 * A.z, w1 * A.w);
+      const float4 in = make_float4(__shfl_up_sync(kAll, far.x, 1), __shfl_up_sync(kAll, far.y, 1),
+                                    __shfl_up_sync(kAll, far.z, 1), __shfl_up_sync(kAll, far.w, 1));
+      if (!act) continue;
+      if (take) near = make_float4(near.x + in.x, near.y + in.y, near.z + in.z, near.w + in.w);
+      const long long q = q0 + ((long long)a * g.n + b) * g.n;
+      atomicAdd(acc + q, near);
+      if (!give) atomicAdd(acc + q + 1, far);
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const long long q = cid(g.n, T.i0[0] + a, T.i0[1] + b, T.i0[2] + e);
-        const float w = corner_w(T, a, b, e);
-        atomicAdd(acc + q, make_float4(w * A.x, w * A.y, w * A.z, w * A.w));
-        const float4 v = pk[q];
+        const float4 v = pk[q + e];
         const float s = A.x * v.x + A.y * v.y + A.z * v.z + A.w * v.w;
 #pragma unroll
         for (int ax = 0; ax < 3; ++ax) gX[ax] += corner_dw(T, ax, a, b, e) * s;
       }
+    }
+  if (!act) return;
   const float4 own = make_float4(T.cl[0] ? 0.0f : -g.dt_dx * gX[0], T.cl[1] ? 0.0f : -g.dt_dx * gX[1],
                                  T.cl[2] ? 0.0f : -g.dt_dx * gX[2], 0.0f);
   atomicAdd(acc + c, own);
@@ -468,6 +686,7 @@ struct mpm_gas {
   Geo g{};
   cudaStream_t stream = nullptr, cstream = nullptr;
   int nfluid = 0;
+  int sms = 1;
   uint8_t* solid = nullptr;
   uint8_t* nbr = nullptr;  // neighbour bits of every cell
   float* states = nullptr;  // (max_steps + 1) x 4 n^3: u (3), d
@@ -476,6 +695,7 @@ struct mpm_gas {
   float* pack = nullptr;  // 4 n^3: packed fields (float4 per cell) of the step being advected
   double* sum = nullptr;
   float* mean = nullptr;
+  int* err = nullptr;  // set by a kernel whose bounded wait ran out
   int step = 0;
   bool started = false, seeds = false;
   long long launches = 0;
@@ -510,6 +730,49 @@ void sweep(const Geo& g, const float* p_in, float* p_out, const float* rhs, cons
   }
 }
 
+// The projection's sweeps from p = 0, in pairs from the size on where those are
+// faster (figures at jacobi2_kernel); returns the buffer that holds the result and adds the
+// launches.
+constexpr int kPairFrom = 160;
+PairShape pair_shape(int n, int sms) {
+  PairShape q;
+  q.tx = n / 4;
+  q.rows = std::min(16, 1024 / q.tx);
+  q.strips = (n + q.rows - 3) / (q.rows - 2);
+  // planes per CTA: the fewest waves x (planes + halo)
+  q.seg = n;
+  for (int k = 1, best = 1 << 30; k <= n / 8; ++k) {
+    const int planes = (n + k - 1) / k, ctas = q.strips * ((n + planes - 1) / planes);
+    const int cost = (ctas + sms - 1) / sms * (planes + 3);
+    if (cost < best) best = cost, q.seg = planes;
+  }
+  q.grid_i = (n + q.seg - 1) / q.seg;
+  q.smem = sizeof(float4) * ((size_t)3 * q.rows * q.tx + kStages * pair_stage_f4(q.tx, q.rows));
+  return q;
+}
+
+float* sweeps(gas_h h, const float* rhs, const float* mean, cudaStream_t st, long long* launches) {
+  const Geo& g = h->g;
+  float* pa = h->p0;
+  float* pb = h->p1;
+  int done = 0;
+  const bool pairs = g.n % 4 == 0 && g.n >= kPairFrom;
+  const PairShape q = pairs ? pair_shape(g.n, h->sms) : PairShape{};
+  while (done < h->cfg.jacobi_iters) {
+    if (pairs && h->cfg.jacobi_iters - done >= 2) {
+      jacobi2_kernel<<<dim3(q.strips, q.grid_i), dim3(q.tx, q.rows), q.smem, st>>>(g, pa, pb, rhs, h->nbr, mean,
+                                                                                  done == 0, q.seg, h->err);
+      done += 2;
+    } else {
+      sweep(g, pa, pb, rhs, h->nbr, mean, done == 0, st);
+      done += 1;
+    }
+    *launches += 1;
+    std::swap(pa, pb);
+  }
+  return pa;
+}
+
 float* state_ptr(gas_h h, int s) { return h->states + (size_t)s * 4 * h->g.n3; }
 
 // Launches of one forward step s -> s + 1 on stream st; returns the launch count.
@@ -526,17 +789,10 @@ long long enqueue_forward(gas_h h, int s, cudaStream_t st) {
   cudaMemsetAsync(h->sum, 0, sizeof(double), st);
   divergence_kernel<<<gr, kCellBlock, 0, st>>>(g, h->un, h->nbr, h->b, h->sum);
   mean_kernel<<<1, 1, 0, st>>>(h->sum, inv_nf, h->mean);
-  float* pa = h->p0;
-  float* pb = h->p1;
-  for (int it = 0; it < h->cfg.jacobi_iters; ++it) {
-    sweep(g, pa, pb, h->b, h->nbr, h->mean, it == 0, st);
-    float* t = pa;
-    pa = pb;
-    pb = t;
-  }
-  gradient_kernel<<<gr, kCellBlock, 0, st>>>(g, pa, h->nbr, h->un);
-  cudaMemcpyAsync(out, h->un, sizeof(float) * 3 * n3, cudaMemcpyDeviceToDevice, st);
-  return 5 + h->cfg.jacobi_iters;
+  long long swept = 0;
+  const float* pa = sweeps(h, h->b, h->mean, st, &swept);
+  gradient_kernel<<<gr, kCellBlock, 0, st>>>(g, pa, h->nbr, h->un, out);
+  return 5 + swept;
 }
 
 // Launches of the adjoint of step s (adj holds the adjoint of state s + 1,
@@ -550,21 +806,12 @@ long long enqueue_backward(gas_h h, int s, cudaStream_t st) {
   float* v = h->adj;  // u (3 n^3), d (n^3)
   // projection: ubar_pre = v - D^T M J G^T v
   gradient_t_kernel<<<gr, kCellBlock, 0, st>>>(g, v, h->nbr, h->b);
-  float* pa = h->p0;
-  float* pb = h->p1;
-  for (int it = 0; it < h->cfg.jacobi_iters; ++it) {
-    sweep(g, pa, pb, h->b, h->nbr, nullptr, it == 0, st);
-    float* t = pa;
-    pa = pb;
-    pb = t;
-  }
+  long long swept = 0;
+  const float* pa = sweeps(h, h->b, nullptr, st, &swept);
   cudaMemsetAsync(h->sum, 0, sizeof(double), st);
   fluid_sum_kernel<<<gr, kCellBlock, 0, st>>>(g, pa, h->nbr, h->sum);
   mean_kernel<<<1, 1, 0, st>>>(h->sum, inv_nf, h->mean);
   divergence_t_kernel<<<gr, kCellBlock, 0, st>>>(g, v, pa, h->nbr, h->mean, h->adj2);
-  // the density output is not projected; its adjoint passes the solid mask
-  cudaMemcpyAsync(h->adj2 + 3 * n3, v + 3 * n3, sizeof(float) * n3, cudaMemcpyDeviceToDevice, st);
-  mask_kernel<<<gr, kCellBlock, 0, st>>>(g, h->nbr, h->adj2 + 3 * n3, 1);
   // advection and buoyancy, from the packed fields of step s
   float4* pk = reinterpret_cast<float4*>(h->pack);
   pack_kernel<<<gr, kCellBlock, 0, st>>>(g, in, in + 3 * n3, pk);
@@ -572,7 +819,7 @@ long long enqueue_backward(gas_h h, int s, cudaStream_t st) {
   cudaMemsetAsync(acc, 0, sizeof(float4) * n3, st);
   advect_t_kernel<<<gr, kCellBlock, 0, st>>>(g, pk, h->nbr, h->adj2, h->adj2 + 3 * n3, acc);
   finish_t_kernel<<<gr, kCellBlock, 0, st>>>(g, acc, h->nbr, h->adj, h->adj + 3 * n3);
-  return 8 + h->cfg.jacobi_iters;
+  return 7 + swept;
 }
 
 sim_status run_graph(gas_h h, std::vector<cudaGraphExec_t>& cache, std::vector<long long>& counts, int s,
@@ -595,9 +842,17 @@ sim_status run_graph(gas_h h, std::vector<cudaGraphExec_t>& cache, std::vector<l
 }
 
 sim_status sync(gas_h h, const char* where) {
-  cudaError_t e = cudaStreamSynchronize(h->stream);
+  int bad = 0;
+  cudaError_t e = cudaMemcpyAsync(&bad, h->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  const cudaError_t es = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess) e = es;
   if (e == cudaSuccess) e = cudaGetLastError();
-  return e == cudaSuccess ? SIM_OK : gcuda(h, e, where);
+  if (e != cudaSuccess) return gcuda(h, e, where);
+  if (bad) {
+    cudaMemset(h->err, 0, sizeof(int));
+    return gfail(h, SIM_E_TIMEOUT, std::string(where) + ": device wait timed out");
+  }
+  return SIM_OK;
 }
 
 cudaError_t copy_in(gas_h h, void* dst, const void* src, size_t bytes, int on_device) {
@@ -629,7 +884,10 @@ sim_status gas_create(const gas_config* cfg, const uint8_t* solid, gas_h* out) {
   h->stream = static_cast<cudaStream_t>(cfg->cuda_stream);
   const size_t n3 = (size_t)g.n3;
   for (size_t c = 0; c < n3; ++c) h->nfluid += solid[c] ? 0 : 1;
-  bool ok = cudaStreamCreateWithFlags(&h->cstream, cudaStreamNonBlocking) == cudaSuccess;
+  int dev = 0;
+  bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+  ok = ok && cudaStreamCreateWithFlags(&h->cstream, cudaStreamNonBlocking) == cudaSuccess;
   ok = ok && cudaMalloc(&h->solid, n3) == cudaSuccess;
   ok = ok && cudaMalloc(&h->nbr, n3) == cudaSuccess;
   ok = ok && cudaMalloc(&h->states, sizeof(float) * 4 * n3 * (size_t)(cfg->max_steps + 1)) == cudaSuccess;
@@ -638,6 +896,10 @@ sim_status gas_create(const gas_config* cfg, const uint8_t* solid, gas_h* out) {
   for (int q = 0; q < 8 && ok; ++q) ok = cudaMalloc(bufs[q], sizeof(float) * sizes[q]) == cudaSuccess;
   ok = ok && cudaMalloc(&h->sum, sizeof(double)) == cudaSuccess;
   ok = ok && cudaMalloc(&h->mean, sizeof(float)) == cudaSuccess;
+  ok = ok && cudaMalloc(&h->err, sizeof(int)) == cudaSuccess && cudaMemset(h->err, 0, sizeof(int)) == cudaSuccess;
+  if (ok && n % 4 == 0 && n >= kPairFrom)
+    ok = cudaFuncSetAttribute(jacobi2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              int(pair_shape(n, h->sms).smem)) == cudaSuccess;
   ok = ok && cudaMemcpy(h->solid, solid, n3, cudaMemcpyHostToDevice) == cudaSuccess;
   if (ok) {
     neighbours_kernel<<<cell_grid(n), kCellBlock>>>(n, h->solid, h->nbr);
@@ -663,8 +925,8 @@ sim_status gas_destroy(gas_h h) {
     if (e) cudaGraphExecDestroy(e);
   for (auto e : h->bwd)
     if (e) cudaGraphExecDestroy(e);
-  void* ptrs[13] = {h->solid, h->nbr, h->states, h->un, h->b, h->p0, h->p1, h->adj, h->adj2, h->acc, h->sum,
-                    h->mean, h->pack};
+  void* ptrs[14] = {h->solid, h->nbr, h->states, h->un, h->b, h->p0, h->p1, h->adj, h->adj2, h->acc, h->sum,
+                    h->mean, h->pack, h->err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (h->cstream) cudaStreamDestroy(h->cstream);
