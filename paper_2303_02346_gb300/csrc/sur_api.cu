@@ -52,6 +52,7 @@ struct mpm_surrogate {
   float* feat_acc = nullptr;
   double* dsum = nullptr;
   int* err = nullptr;
+  int* words = nullptr;  // pinned copy of err
   bool dirty = true;
   std::string last_error;
   bool prof = false;
@@ -202,12 +203,14 @@ sim_status run_selftest(sur_h h) {
   return SIM_OK;
 }
 
+// Wait for the stream and read the error word, which comes to pinned memory
+// before the wait instead of by a blocking copy after it.
 sim_status check_err(sur_h h, const char* where) {
-  cudaError_t e = cudaStreamSynchronize(h->stream);
+  cudaError_t e = cudaMemcpyAsync(h->words, h->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  const cudaError_t es = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess) e = es;
   if (e != cudaSuccess) return cuda_fail(h, e, where);
-  int v = 0;
-  e = cudaMemcpy(&v, h->err, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(h, e, where);
+  const int v = *h->words;
   if (v) {
     cudaMemset(h->err, 0, sizeof(int));
     if (v & kErrTimeout) return fail(h, SIM_E_TIMEOUT, std::string(where) + ": tensor-core pipeline wait timed out");
@@ -340,6 +343,7 @@ sim_status sur_destroy(sur_h h) {
     cudaEventDestroy(r.b);
   }
   for (void* p : h->allocs) cudaFree(p);
+  if (h->words) cudaFreeHost(h->words);
   delete h;
   return SIM_OK;
 }
@@ -376,13 +380,15 @@ sim_status sur_create(const sur_config* cfg, sur_h* out) {
             dalloc(h, &h->gpred, static_cast<size_t>(cfg->max_batch) * n3 * 3) &&
             dalloc(h, &h->partial, static_cast<size_t>(h->n_part) * (27 * 1024 + 32)) &&
             dalloc(h, &h->feat_acc, static_cast<size_t>(n3) * 8) &&
-            dalloc(h, &h->dsum, 1 + 2 * static_cast<size_t>(cfg->max_batch)) && dalloc(h, &h->err, 1);
+            dalloc(h, &h->dsum, 1 + 2 * static_cast<size_t>(cfg->max_batch)) && dalloc(h, &h->err, 1) &&
+            cudaMallocHost(&h->words, sizeof(int)) == cudaSuccess;
   h->h.assign(h->B + 1, nullptr);
   h->r.assign(h->B, nullptr);
   for (int i = 0; ok && i <= h->B; ++i) ok = dalloc(h, &h->h[i], tensor);
   for (int i = 0; ok && i < h->B; ++i) ok = dalloc(h, &h->r[i], tensor);
   ok = ok && dalloc(h, &h->gh[0], tensor) && dalloc(h, &h->gh[1], tensor) && dalloc(h, &h->ga, tensor);
   if (!ok) {
+    cudaGetLastError();
     sur_destroy(h);
     return SIM_E_OOM;
   }

@@ -91,6 +91,16 @@ __device__ __forceinline__ bool make_stencil(const float* x, int n, Stencil& s) 
   return ok;
 }
 
+// four consecutive floats (16-byte aligned) reduced into memory at once
+__device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float c, float d) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
+               : "memory");
+}
+
+// Bound by L2's reductions (the caller's particle order is arbitrary, so the 27
+// nodes of neighbouring threads share nothing): the mass and the momentum go
+// out as one vector reduction, the material's mass as a scalar, 2 a node
+// instead of 5 (100k particles on 64^3: 124 -> 47 us).
 __global__ void features_scatter_kernel(FeatArgs a, const float* __restrict__ x, const float* __restrict__ v,
                                         const float* __restrict__ C, const uint8_t* __restrict__ mat,
                                         float* acc, int* err) {
@@ -126,10 +136,9 @@ __global__ void features_scatter_kernel(FeatArgs a, const float* __restrict__ x,
         const long long node =
             (static_cast<long long>(s.base[0] + oi) * n + (s.base[1] + oj)) * n + (s.base[2] + ok);
         float* dst = acc + node * 8;
-        atomicAdd(dst + 0, wm);
-        atomicAdd(dst + 1, wm * (vp[0] + Cp[0] * d0 + Cp[1] * d1 + Cp[2] * d2));
-        atomicAdd(dst + 2, wm * (vp[1] + Cp[3] * d0 + Cp[4] * d1 + Cp[5] * d2));
-        atomicAdd(dst + 3, wm * (vp[2] + Cp[6] * d0 + Cp[7] * d1 + Cp[8] * d2));
+        red_add_v4(dst, wm, wm * (vp[0] + Cp[0] * d0 + Cp[1] * d1 + Cp[2] * d2),
+                   wm * (vp[1] + Cp[3] * d0 + Cp[4] * d1 + Cp[5] * d2),
+                   wm * (vp[2] + Cp[6] * d0 + Cp[7] * d1 + Cp[8] * d2));
         if (mt < 3) atomicAdd(dst + 4 + mt, wm);
       }
 }
@@ -201,7 +210,9 @@ __global__ void features_vjp_kernel(FeatArgs a, const float* __restrict__ x, con
   float gv[3] = {0.f, 0.f, 0.f}, gC[9], gx[3] = {0.f, 0.f, 0.f};
 #pragma unroll
   for (int k = 0; k < 9; ++k) gC[k] = 0.0f;
+#pragma unroll
   for (int oi = 0; oi < 3; ++oi)
+#pragma unroll
     for (int oj = 0; oj < 3; ++oj)
 #pragma unroll
       for (int ok = 0; ok < 3; ++ok) {
@@ -247,35 +258,54 @@ __device__ __forceinline__ void split_node(const SurGeom& g, long long v, int& i
 }
 
 // ---------------------------------------------------------------------------
-// lift: h0 = bf16(W_l f + b_l) at every interior row
+// lift: h0 = bf16(W_l f + b_l) at every interior row. Memory moves 80 bytes a
+// node; the weights' shared-memory loads were the bound (one word per product),
+// so a thread takes two nodes and reads the weights 16 bytes at a time.
+// 8 frames of 64^3: 46 -> 39 us.
 // ---------------------------------------------------------------------------
-__global__ void lift_kernel(SurGeom g, const uint16_t* __restrict__ frames, const int* __restrict__ idx,
-                            const float* __restrict__ wl, const float* __restrict__ bl, __nv_bfloat16* h0) {
-  __shared__ float sw[32 * 8 + 32];
+__global__ void __launch_bounds__(256) lift_kernel(SurGeom g, const uint16_t* __restrict__ frames,
+                                                   const int* __restrict__ idx, const float* __restrict__ wl,
+                                                   const float* __restrict__ bl, __nv_bfloat16* h0) {
+  __shared__ float4 sw4[64 + 8];
+  float* sw = reinterpret_cast<float*>(sw4);
   for (int i = threadIdx.x; i < 256 + 32; i += blockDim.x) sw[i] = i < 256 ? rbf(wl[i]) : bl[i - 256];
   __syncthreads();
   const int b = blockIdx.y;
   const long long n3 = static_cast<long long>(g.n) * g.n * g.n;
   const long long fr = idx ? idx[b] : b;
-  for (long long vtx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; vtx < n3;
-       vtx += static_cast<long long>(gridDim.x) * blockDim.x) {
-    float f[8];
-    unpack8(reinterpret_cast<const uint4*>(frames)[fr * n3 + vtx], f);
+  const long long step = static_cast<long long>(gridDim.x) * blockDim.x;
+  for (long long v0 = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; v0 < n3; v0 += 2 * step) {
+    const long long v1 = v0 + step;
+    const bool two = v1 < n3;
+    const uint4 r0 = reinterpret_cast<const uint4*>(frames)[fr * n3 + v0];
+    const uint4 r1 = two ? reinterpret_cast<const uint4*>(frames)[fr * n3 + v1] : r0;
+    float f[2][8];
+    unpack8(r0, f[0]);
+    unpack8(r1, f[1]);
     int i, j, k;
-    split_node(g, vtx, i, j, k);
-    const long long row = pad_row(g, b, i, j, k);
+    split_node(g, v0, i, j, k);
+    const long long row0 = pad_row(g, b, i, j, k);
+    split_node(g, two ? v1 : v0, i, j, k);
+    const long long row1 = pad_row(g, b, i, j, k);
 #pragma unroll 1
     for (int c = 0; c < 4; ++c) {
-      float o[8];
+      float o0[8], o1[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const int oc = c * 8 + e;
-        float s = sw[256 + oc];
+        const float4 wa = sw4[oc * 2], wb = sw4[oc * 2 + 1];
+        const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+        float s0 = sw[256 + oc], s1 = s0;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) s += sw[oc * 8 + q] * f[q];
-        o[e] = s;
+        for (int q = 0; q < 8; ++q) {
+          s0 += w[q] * f[0][q];
+          s1 += w[q] * f[1][q];
+        }
+        o0[e] = s0;
+        o1[e] = s1;
       }
-      *reinterpret_cast<uint4*>(h0 + (c * g.plane + row) * 8) = pack8(o);
+      *reinterpret_cast<uint4*>(h0 + (c * g.plane + row0) * 8) = pack8(o0);
+      if (two) *reinterpret_cast<uint4*>(h0 + (c * g.plane + row1) * 8) = pack8(o1);
     }
   }
 }
@@ -285,9 +315,16 @@ __global__ void lift_kernel(SurGeom g, const uint16_t* __restrict__ frames, cons
 // (BF16), dL/dW_p, dL/db_p and per-frame error sums
 // ---------------------------------------------------------------------------
 constexpr int kProjThreads = 256;
+constexpr int kRowWords = 17;  // words per node of a transposed channel row (16 of two BF16, one of padding)
 
+// One thread per node. A warp's nodes are summed into dL/dW_p through a
+// transpose in its own shared memory: each lane leaves its node's 32 channels
+// there and takes one channel of all 32 nodes, so that a lane accumulates 3
+// entries instead of 96 (which took 255 registers and spills); no barrier.
+// The weights are read 16 bytes at a time. 8 frames of 64^3: training 164 -> 102
+// us, inference 67 -> 46.
 template <int MODE>
-__global__ void __launch_bounds__(kProjThreads) proj_kernel(SurGeom g, int batch,
+__global__ void __launch_bounds__(kProjThreads, (MODE & 2) ? 2 : (MODE & 4) ? 3 : 4) proj_kernel(SurGeom g, int batch,
                                                             const uint16_t* __restrict__ frames,
                                                             const int* __restrict__ idx,
                                                             const int* __restrict__ tgt,
@@ -296,109 +333,131 @@ __global__ void __launch_bounds__(kProjThreads) proj_kernel(SurGeom g, int batch
                                                             const float* __restrict__ bp, float* pred,
                                                             __nv_bfloat16* g_h, float* g_pred, float* grad_wp,
                                                             double* loss_acc, double* frame_sums) {
-  __shared__ float sw[96 + 3];
+  constexpr bool want_grad = MODE & 2, want_sums = MODE & 4, given = MODE & 8;
+  constexpr unsigned kAll = 0xffffffffu;
+  __shared__ float4 sw4[24 + 1];
   __shared__ float red[kProjThreads / 32][101];
+  __shared__ uint32_t rows[want_grad ? kProjThreads * kRowWords : 1];
+  __shared__ float4 grads[want_grad ? kProjThreads : 1];
+  float* sw = reinterpret_cast<float*>(sw4);
   for (int i = threadIdx.x; i < 99; i += blockDim.x) sw[i] = i < 96 ? rbf(wp[i]) : bp[i - 96];
   __syncthreads();
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int b = blockIdx.y;
   const long long n3 = static_cast<long long>(g.n) * g.n * g.n;
   const long long fr = idx ? idx[b] : b;
   const long long ft = tgt ? tgt[b] : 0;
   const float inv_count = 1.0f / (static_cast<float>(batch) * static_cast<float>(n3) * 3.0f);
-  constexpr bool want_grad = MODE & 2, want_sums = MODE & 4, given = MODE & 8;
-  float gw[96], gb[3], l2 = 0.f, t2 = 0.f;
-  if (want_grad) {
+  float gw[3] = {0.f, 0.f, 0.f}, gb[3] = {0.f, 0.f, 0.f}, l2 = 0.f, t2 = 0.f;
+  for (long long base = blockIdx.x * static_cast<long long>(blockDim.x); base < n3;
+       base += static_cast<long long>(gridDim.x) * blockDim.x) {
+    const long long vtx = base + threadIdx.x;
+    const bool in = vtx < n3;
+    float gp[3] = {0.f, 0.f, 0.f};
+    uint4 raw[4] = {};
+    if (in) {
+      int i, j, k;
+      split_node(g, vtx, i, j, k);
+      const long long row = pad_row(g, b, i, j, k);
 #pragma unroll
-    for (int i = 0; i < 96; ++i) gw[i] = 0.f;
-    gb[0] = gb[1] = gb[2] = 0.f;
-  }
-  for (long long vtx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; vtx < n3;
-       vtx += static_cast<long long>(gridDim.x) * blockDim.x) {
-    int i, j, k;
-    split_node(g, vtx, i, j, k);
-    const long long row = pad_row(g, b, i, j, k);
-    float hv[32];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float t[8];
-      unpack8(*reinterpret_cast<const uint4*>(h + (c * g.plane + row) * 8), t);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) hv[c * 8 + e] = t[e];
-    }
-    float f[8];
-    unpack8(reinterpret_cast<const uint4*>(frames)[fr * n3 + vtx], f);
-    float p[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      float s = sw[96 + c];
-#pragma unroll
-      for (int o = 0; o < 32; ++o) s += sw[c * 32 + o] * hv[o];
-      p[c] = f[1 + c] + s;
-    }
-    if (MODE & 1) {
-      float* dst = pred + (static_cast<long long>(b) * n3 + vtx) * 3;
-      dst[0] = p[0];
-      dst[1] = p[1];
-      dst[2] = p[2];
-    }
-    if (given) {
-      // cotangent of the prediction supplied by the caller: dL/dh only
-      const float* gp = g_pred + (static_cast<long long>(b) * n3 + vtx) * 3;
+      for (int c = 0; c < 4; ++c) raw[c] = *reinterpret_cast<const uint4*>(h + (c * g.plane + row) * 8);
+      const uint4 fraw = reinterpret_cast<const uint4*>(frames)[fr * n3 + vtx];
+      float p[3] = {sw[96], sw[97], sw[98]};
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        float o8[8];
+        float hv[8];
+        unpack8(raw[c], hv);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const int o = c * 8 + e;
-          o8[e] = sw[o] * gp[0] + sw[32 + o] * gp[1] + sw[64 + o] * gp[2];
+        for (int m = 0; m < 3; ++m) {
+          const float4 wa = sw4[m * 8 + c * 2], wb = sw4[m * 8 + c * 2 + 1];
+          const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+          for (int e = 0; e < 8; ++e) p[m] += w[e] * hv[e];
         }
-        *reinterpret_cast<uint4*>(g_h + (c * g.plane + row) * 8) = pack8(o8);
       }
-    }
-    if (want_grad || want_sums) {
-      float tf[8];
-      unpack8(reinterpret_cast<const uint4*>(frames)[ft * n3 + vtx], tf);
-      float d[3] = {p[0] - tf[1], p[1] - tf[2], p[2] - tf[3]};
-      l2 += d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-      t2 += tf[1] * tf[1] + tf[2] * tf[2] + tf[3] * tf[3];
-      if (want_grad) {
-        float gp[3];
+      float f[8];
+      unpack8(fraw, f);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          gp[c] = 2.0f * d[c] * inv_count;
-          gb[c] += gp[c];
+      for (int m = 0; m < 3; ++m) p[m] = f[1 + m] + p[m];
+      if (MODE & 1) {
+        float* dst = pred + (static_cast<long long>(b) * n3 + vtx) * 3;
+        dst[0] = p[0];
+        dst[1] = p[1];
+        dst[2] = p[2];
+      }
+      if (given) {
+        // cotangent of the prediction supplied by the caller: dL/dh only
+        const float* src = g_pred + (static_cast<long long>(b) * n3 + vtx) * 3;
 #pragma unroll
-          for (int o = 0; o < 32; ++o) gw[c * 32 + o] += gp[c] * hv[o];
+        for (int m = 0; m < 3; ++m) gp[m] = src[m];
+      }
+      if (want_grad || want_sums) {
+        float tf[8];
+        unpack8(reinterpret_cast<const uint4*>(frames)[ft * n3 + vtx], tf);
+        const float d[3] = {p[0] - tf[1], p[1] - tf[2], p[2] - tf[3]};
+        l2 += d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+        t2 += tf[1] * tf[1] + tf[2] * tf[2] + tf[3] * tf[3];
+        if (want_grad) {
+#pragma unroll
+          for (int m = 0; m < 3; ++m) {
+            gp[m] = 2.0f * d[m] * inv_count;
+            gb[m] += gp[m];
+          }
+          if (g_pred) {
+            float* dst = g_pred + (static_cast<long long>(b) * n3 + vtx) * 3;
+            dst[0] = gp[0];
+            dst[1] = gp[1];
+            dst[2] = gp[2];
+          }
         }
-        if (g_pred) {
-          float* dst = g_pred + (static_cast<long long>(b) * n3 + vtx) * 3;
-          dst[0] = gp[0];
-          dst[1] = gp[1];
-          dst[2] = gp[2];
-        }
+      }
+      if (want_grad || given) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
+          const float4 a0 = sw4[c * 2], a1 = sw4[c * 2 + 1], b0 = sw4[8 + c * 2], b1 = sw4[8 + c * 2 + 1],
+                       c0 = sw4[16 + c * 2], c1 = sw4[16 + c * 2 + 1];
+          const float wa[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+          const float wb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+          const float wc[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
           float o8[8];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const int o = c * 8 + e;
-            o8[e] = sw[o] * gp[0] + sw[32 + o] * gp[1] + sw[64 + o] * gp[2];
-          }
+          for (int e = 0; e < 8; ++e) o8[e] = wa[e] * gp[0] + wb[e] * gp[1] + wc[e] * gp[2];
           *reinterpret_cast<uint4*>(g_h + (c * g.plane + row) * 8) = pack8(o8);
         }
       }
     }
-  }
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  if (want_grad) {
-#pragma unroll 4
-    for (int i = 0; i < 96; ++i) {
-      const float s = warp_sum(gw[i]);
-      if (lane == 0) red[warp][i] = s;
+    if (want_grad) {
+      // lanes past the last node leave zeros
+      uint32_t* mine = rows + threadIdx.x * kRowWords;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        mine[c * 4] = raw[c].x;
+        mine[c * 4 + 1] = raw[c].y;
+        mine[c * 4 + 2] = raw[c].z;
+        mine[c * 4 + 3] = raw[c].w;
+      }
+      grads[threadIdx.x] = make_float4(gp[0], gp[1], gp[2], 0.f);
+      __syncwarp();
+      const uint32_t* col = rows + warp * 32 * kRowWords + lane / 2;
+      const float4* gr = grads + warp * 32;
+#pragma unroll 8
+      for (int r = 0; r < 32; ++r) {
+        const uint32_t w2 = col[r * kRowWords];
+        const float hv = __uint_as_float((lane & 1) ? (w2 & 0xffff0000u) : (w2 << 16));
+        const float4 q = gr[r];
+        gw[0] += q.x * hv;
+        gw[1] += q.y * hv;
+        gw[2] += q.z * hv;
+      }
+      __syncwarp();
     }
-    for (int c = 0; c < 3; ++c) {
-      const float s = warp_sum(gb[c]);
-      if (lane == 0) red[warp][96 + c] = s;
+  }
+  if (want_grad) {
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      red[warp][m * 32 + lane] = gw[m];
+      const float s = warp_sum(gb[m]);
+      if (lane == 0) red[warp][96 + m] = s;
     }
   }
   const float sl = warp_sum(l2), st = warp_sum(t2);
@@ -427,7 +486,11 @@ __global__ void __launch_bounds__(kProjThreads) proj_kernel(SurGeom g, int batch
 }
 
 // ---------------------------------------------------------------------------
-// lift backward: dW_l, db_l and optionally dL/dframe
+// lift backward: dW_l, db_l and optionally dL/dframe. As in the projection, a
+// warp's nodes pass through its own shared memory, and lane o sums the 8
+// entries of output channel o (and its bias) over the 32 nodes: 3 shared loads
+// for 9 sums, where one entry a thread took 2 loads a sum behind two barriers
+// per 256 nodes. 8 frames of 64^3: 162 -> 60 us.
 // ---------------------------------------------------------------------------
 constexpr int kLbThreads = 256;
 
@@ -439,44 +502,41 @@ __global__ void __launch_bounds__(kLbThreads) lift_bwd_kernel(SurGeom g, int bat
                                                               const float* __restrict__ g_pred, float* grad_wl,
                                                               float* grad_bl, float* g_frames) {
   __shared__ float sw[256];
-  __shared__ float sg[kLbThreads][33];
-  __shared__ float sf[kLbThreads][9];
+  __shared__ uint32_t rows[kLbThreads * kRowWords];
+  __shared__ float4 sf[kLbThreads * 2];
   for (int i = threadIdx.x; i < 256; i += blockDim.x) sw[i] = rbf(wl[i]);
+  __syncthreads();
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int b = blockIdx.y;
   const long long n3 = static_cast<long long>(g.n) * g.n * g.n;
   const long long fr = idx ? idx[b] : b;
-  const int o_me = threadIdx.x / 8, q_me = threadIdx.x % 8;  // (o, q) pair of this thread's dW_l entry
-  float accw = 0.f, accb = 0.f;
+  float accw[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, accb = 0.f;
   const long long step = static_cast<long long>(gridDim.x) * blockDim.x;
   for (long long base = blockIdx.x * static_cast<long long>(blockDim.x); base < n3; base += step) {
     const long long vtx = base + threadIdx.x;
-    __syncthreads();
+    uint4 raw[4] = {};  // lanes past the last node leave zeros
+    float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (vtx < n3) {
       int i, j, k;
       split_node(g, vtx, i, j, k);
       const long long row = pad_row(g, b, i, j, k);
-      float gv[32];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        float t[8];
-        unpack8(*reinterpret_cast<const uint4*>(gh + (c * g.plane + row) * 8), t);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) gv[c * 8 + e] = t[e];
-      }
-      float f[8];
+      for (int c = 0; c < 4; ++c) raw[c] = *reinterpret_cast<const uint4*>(gh + (c * g.plane + row) * 8);
       unpack8(reinterpret_cast<const uint4*>(frames)[fr * n3 + vtx], f);
-#pragma unroll
-      for (int o = 0; o < 32; ++o) sg[threadIdx.x][o] = gv[o];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) sf[threadIdx.x][q] = f[q];
       if (g_frames) {
-        float gf[8];
+        float gf[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          float s = 0.f;
+        for (int c = 0; c < 4; ++c) {
+          float gv[8];
+          unpack8(raw[c], gv);
 #pragma unroll
-          for (int o = 0; o < 32; ++o) s += sw[o * 8 + q] * gv[o];
-          gf[q] = s;
+          for (int e = 0; e < 8; ++e) {
+            const float4 wa = reinterpret_cast<const float4*>(sw)[(c * 8 + e) * 2],
+                         wb = reinterpret_cast<const float4*>(sw)[(c * 8 + e) * 2 + 1];
+            const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+            for (int q = 0; q < 8; ++q) gf[q] += w[q] * gv[e];
+          }
         }
         const float* gp = g_pred + (static_cast<long long>(b) * n3 + vtx) * 3;
         gf[1] += gp[0];
@@ -486,19 +546,52 @@ __global__ void __launch_bounds__(kLbThreads) lift_bwd_kernel(SurGeom g, int bat
         dst[0] = make_float4(gf[0], gf[1], gf[2], gf[3]);
         dst[1] = make_float4(gf[4], gf[5], gf[6], gf[7]);
       }
-    } else {
-#pragma unroll
-      for (int o = 0; o < 32; ++o) sg[threadIdx.x][o] = 0.f;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) sf[threadIdx.x][q] = 0.f;
     }
-    __syncthreads();
-    for (int r = 0; r < kLbThreads; ++r) accw += sg[r][o_me] * sf[r][q_me];
-    if (threadIdx.x < 32)
-      for (int r = 0; r < kLbThreads; ++r) accb += sg[r][threadIdx.x];
+    uint32_t* mine = rows + threadIdx.x * kRowWords;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      mine[c * 4] = raw[c].x;
+      mine[c * 4 + 1] = raw[c].y;
+      mine[c * 4 + 2] = raw[c].z;
+      mine[c * 4 + 3] = raw[c].w;
+    }
+    sf[threadIdx.x * 2] = make_float4(f[0], f[1], f[2], f[3]);
+    sf[threadIdx.x * 2 + 1] = make_float4(f[4], f[5], f[6], f[7]);
+    __syncwarp();
+    const uint32_t* col = rows + warp * 32 * kRowWords + lane / 2;
+    const float4* fw = sf + warp * 64;
+#pragma unroll 8
+    for (int r = 0; r < 32; ++r) {
+      const uint32_t w2 = col[r * kRowWords];
+      const float gv = __uint_as_float((lane & 1) ? (w2 & 0xffff0000u) : (w2 << 16));
+      const float4 a = fw[r * 2], c = fw[r * 2 + 1];
+      accw[0] += gv * a.x;
+      accw[1] += gv * a.y;
+      accw[2] += gv * a.z;
+      accw[3] += gv * a.w;
+      accw[4] += gv * c.x;
+      accw[5] += gv * c.y;
+      accw[6] += gv * c.z;
+      accw[7] += gv * c.w;
+      accb += gv;
+    }
+    __syncwarp();
   }
-  atomicAdd(grad_wl + o_me * 8 + q_me, accw);
-  if (threadIdx.x < 32) atomicAdd(grad_bl + threadIdx.x, accb);
+  // over the CTA's warps, then one atomic per entry
+  __syncthreads();
+  float* red = reinterpret_cast<float*>(rows);  // 8 warps x 288
+#pragma unroll
+  for (int q = 0; q < 8; ++q) red[warp * 288 + lane * 8 + q] = accw[q];
+  red[warp * 288 + 256 + lane] = accb;
+  __syncthreads();
+  for (int i = threadIdx.x; i < 288; i += blockDim.x) {
+    float s = 0.f;
+    for (int w = 0; w < kLbThreads / 32; ++w) s += red[w * 288 + i];
+    if (i < 256)
+      atomicAdd(grad_wl + i, s);
+    else
+      atomicAdd(grad_bl + i - 256, s);
+  }
 }
 
 // ---------------------------------------------------------------------------
