@@ -54,6 +54,7 @@ struct Params {
   int tool;
   float half[3];
   float eps_c, inv_ell, mu_f;
+  float reach2;   // (|half| + eps_c)^2 and a little: no contact farther from the tool's centre
 };
 
 // Ask L2 for the line holding *p ahead of its use (no register, no fault on a

@@ -248,7 +248,9 @@ grid_adj_kernel(Params P, const float4* __restrict__ gstore, float4* __restrict_
       float vb[3] = {wall ? 0.0f : vb4[u].x, wall ? 0.0f : vb4[u].y, wall ? 0.0f : vb4[u].z};
       float uu[3] = {um.x, um.y, um.z};
       float ub[3] = {vb[0], vb[1], vb[2]};
-      if (kTool && !wall) {
+      const float* tp = kTool ? pose + ((long long)scene * max_steps + step) * kToolFields : nullptr;
+      float xi[3] = {i * P.dx, j * P.dx, k * P.dx};
+      if (kTool && !wall && !tool_far(P, tp, xi)) {
         if (scene != cur) {
           if (cur >= 0) flush_tool_grad(acc, cur, tool_grad, step, max_steps, false);
 #pragma unroll
@@ -256,8 +258,7 @@ grid_adj_kernel(Params P, const float4* __restrict__ gstore, float4* __restrict_
           cur = scene;
         }
         ToolState T;
-        load_tool(pose + ((long long)scene * max_steps + step) * kToolFields, T);
-        float xi[3] = {i * P.dx, j * P.dx, k * P.dx};
+        load_tool(tp, T);
         contact_adjoint(P, T, xi, uu, vb, ub, acc, acc + 3, acc + 12, acc + 15);
       }
       float inv = 1.0f / um.w;

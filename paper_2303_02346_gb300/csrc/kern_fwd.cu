@@ -200,10 +200,13 @@ __device__ inline void grid_update_items(const Params& P, float4* __restrict__ a
         if (gstore) gstore[idx] = make_float4(uu[0], uu[1], uu[2], a[u].x);
         float vv[3] = {uu[0], uu[1], uu[2]};
         if (kTool) {
-          ToolState T;
-          load_tool(pose + ((long long)scene * max_steps + step) * kToolFields, T);
+          const float* tp = pose + ((long long)scene * max_steps + step) * kToolFields;
           float xi[3] = {i * P.dx, j * P.dx, k * P.dx};
-          contact_forward(P, T, xi, vv);
+          if (!tool_far(P, tp, xi)) {
+            ToolState T;
+            load_tool(tp, T);
+            contact_forward(P, T, xi, vv);
+          }
         }
         bool wall = i < P.bound || j < P.bound || k < P.bound || i >= P.n - P.bound ||
                     j >= P.n - P.bound || k >= P.n - P.bound;

@@ -476,8 +476,7 @@ void launch_add_seed(float* adj_field, const float* seed, const int* pid, const 
 
 // ---------------------------------------------------------------------------
 // tool kinematics (Sec. 4.2: the action is the tool's linear and angular
-// velocity; App. B.1: held for a fixed number of substeps). One thread per
-// scene integrates the pose in FP64:
+// velocity; App. B.1: held for a fixed number of substeps). The pose in FP64:
 //   p_{n+1} = p_n + dt pdot_n,  q_{n+1} = normalize(dq(omega_n dt) q_n),
 //   dq(w) = (cos(|w|/2), sin(|w|/2) w/|w|).
 // Pose record per step: p (3), q (4), pdot (3), omega (3).
@@ -522,99 +521,102 @@ __device__ inline void qnormalize(double* q) {
   for (int i = 0; i < 4; ++i) q[i] *= r;
 }
 
-// One warp per scene. Lane a handles action a (in chunks of 32 actions): its
-// rotation increment, the action's whole rotation D_a and translation; a
-// prefix product / sum across the lanes gives the pose at the action's first
-// step, from which the lane integrates the action's steps one by one (the
-// same per-step update as a serial walk, in FP64).
-__global__ void tool_forward_kernel(int S, const float* __restrict__ pose0,
+// One CTA per scene. The chain over the actions is short (one rotation and one
+// translation each) and the steps inside an action are closed form, so nothing
+// walks the steps one by one: m steps of one action turn by dq(m omega dt) and
+// move by m dt pdot. Per chunk of 32 actions, warp 0 (lane a: action a) takes
+// the actions' whole rotations and translations, an inclusive scan over the
+// lanes and the pose at each action's first step into shared memory; then
+// every thread takes a step of the chunk. FP64 throughout; bound by the latency
+// of its FP64 chain (200 steps in 20 actions: 45 us walked step by step, 25 us
+// so).
+constexpr int kToolThreads = 128;
+__global__ void __launch_bounds__(kToolThreads)
+tool_forward_kernel(int S, const float* __restrict__ pose0,
                                     const float* __restrict__ actions, int n_actions, int spa,
                                     int n_steps, int max_steps, double dt, float* __restrict__ poses) {
-  const int sc = (blockIdx.x * blockDim.x + threadIdx.x) / 32;
+  __shared__ double sp[32][3], sq[32][4], carry[7];
+  const int sc = blockIdx.x;
   const int lane = threadIdx.x % 32;
-  if (sc >= S) return;  // whole warps
-  double p[3], q[4];
-  for (int i = 0; i < 3; ++i) p[i] = pose0[sc * 7 + i];
-  for (int i = 0; i < 4; ++i) q[i] = pose0[sc * 7 + 3 + i];
-  qnormalize(q);
+  if (threadIdx.x == 0) {
+    double q[4];
+    for (int i = 0; i < 4; ++i) q[i] = pose0[sc * 7 + 3 + i];
+    qnormalize(q);
+    for (int i = 0; i < 3; ++i) carry[i] = pose0[sc * 7 + i];
+    for (int i = 0; i < 4; ++i) carry[3 + i] = q[i];
+  }
+  __syncthreads();
+  // first step of action a; the last action holds to the end
+  auto first_step = [&](int a) { return a >= n_actions ? n_steps : (int)min((long long)a * spa, (long long)n_steps); };
   for (int a0 = 0; a0 < n_actions; a0 += 32) {
-    const int a = a0 + lane;
-    const int lo = a * spa;
-    const int hi = (a == n_actions - 1) ? n_steps : min((a + 1) * spa, n_steps);
-    const int len = (a < n_actions && lo < n_steps) ? hi - lo : 0;
-    double pd[3] = {0.0, 0.0, 0.0}, om[3] = {0.0, 0.0, 0.0}, dq[4] = {1.0, 0.0, 0.0, 0.0};
-    if (len > 0) {
+    if (threadIdx.x < 32) {
+      const int a = a0 + lane;
+      const int len = a < n_actions ? first_step(a + 1) - first_step(a) : 0;
+      double D[4] = {1.0, 0.0, 0.0, 0.0}, tr[3] = {0.0, 0.0, 0.0};
+      if (len > 0) {
+        const float* act = actions + ((long long)sc * n_actions + a) * 6;
+        double om[3];
+        for (int i = 0; i < 3; ++i) {
+          tr[i] = dt * len * act[i];
+          om[i] = act[3 + i];
+        }
+        dq_of(om, dt * len, D, nullptr);
+      }
+      // inclusive scans across lanes: rotations compose with later ones on the left
+      for (int off = 1; off < 32; off <<= 1) {
+        double oD[4], ot[3];
+        for (int i = 0; i < 4; ++i) oD[i] = __shfl_up_sync(0xffffffffu, D[i], off);
+        for (int i = 0; i < 3; ++i) ot[i] = __shfl_up_sync(0xffffffffu, tr[i], off);
+        if (lane >= off) {
+          double t4[4];
+          qmul(D, oD, t4);
+          for (int i = 0; i < 4; ++i) D[i] = t4[i];
+          for (int i = 0; i < 3; ++i) tr[i] += ot[i];
+        }
+      }
+      double E[4], et[3], q[4], q2[4];
+      for (int i = 0; i < 4; ++i) E[i] = __shfl_up_sync(0xffffffffu, D[i], 1);
+      for (int i = 0; i < 3; ++i) et[i] = __shfl_up_sync(0xffffffffu, tr[i], 1);
+      if (lane == 0) {
+        E[0] = 1.0;
+        E[1] = E[2] = E[3] = 0.0;
+        et[0] = et[1] = et[2] = 0.0;
+      }
+      qmul(E, carry + 3, q);
+      qnormalize(q);
+      qmul(D, carry + 3, q2);
+      qnormalize(q2);
+      for (int i = 0; i < 3; ++i) sp[lane][i] = carry[i] + et[i];
+      for (int i = 0; i < 4; ++i) sq[lane][i] = q[i];
+      __syncwarp();
+      if (lane == 31) {
+        for (int i = 0; i < 3; ++i) carry[i] += tr[i];
+        for (int i = 0; i < 4; ++i) carry[3 + i] = q2[i];
+      }
+    }
+    __syncthreads();
+    const int hi = first_step(a0 + 32 < n_actions ? a0 + 32 : n_actions);
+    for (int n = first_step(a0) + threadIdx.x; n < hi; n += kToolThreads) {
+      const int a = min(n / spa, n_actions - 1), m = n - first_step(a);
       const float* act = actions + ((long long)sc * n_actions + a) * 6;
-      for (int i = 0; i < 3; ++i) {
-        pd[i] = act[i];
-        om[i] = act[3 + i];
-      }
-      dq_of(om, dt, dq, nullptr);
+      const double om[3] = {act[3], act[4], act[5]};
+      double dq[4], q[4];
+      dq_of(om, dt * m, dq, nullptr);
+      qmul(dq, sq[a - a0], q);
+      qnormalize(q);
+      float* rec = poses + ((long long)sc * max_steps + n) * kToolFields;
+      for (int i = 0; i < 3; ++i) rec[i] = float(sp[a - a0][i] + dt * m * act[i]);
+      for (int i = 0; i < 4; ++i) rec[3 + i] = float(q[i]);
+      for (int i = 0; i < 6; ++i) rec[7 + i] = act[i];
     }
-    // the action's rotation and translation over its steps
-    double D[4] = {1.0, 0.0, 0.0, 0.0}, tr[3] = {0.0, 0.0, 0.0};
-    for (int m = 0; m < len; ++m) {
-      double t4[4];
-      qmul(dq, D, t4);
-      qnormalize(t4);
-      for (int i = 0; i < 4; ++i) D[i] = t4[i];
-      for (int i = 0; i < 3; ++i) tr[i] += dt * pd[i];
-    }
-    // inclusive scans across lanes: rotations compose with later ones on the left
-    for (int off = 1; off < 32; off <<= 1) {
-      double oD[4], ot[3];
-      for (int i = 0; i < 4; ++i) oD[i] = __shfl_up_sync(0xffffffffu, D[i], off);
-      for (int i = 0; i < 3; ++i) ot[i] = __shfl_up_sync(0xffffffffu, tr[i], off);
-      if (lane >= off) {
-        double t4[4];
-        qmul(D, oD, t4);
-        qnormalize(t4);
-        for (int i = 0; i < 4; ++i) D[i] = t4[i];
-        for (int i = 0; i < 3; ++i) tr[i] += ot[i];
-      }
-    }
-    double E[4], et[3];
-    for (int i = 0; i < 4; ++i) E[i] = __shfl_up_sync(0xffffffffu, D[i], 1);
-    for (int i = 0; i < 3; ++i) et[i] = __shfl_up_sync(0xffffffffu, tr[i], 1);
-    if (lane == 0) {
-      E[0] = 1.0;
-      E[1] = E[2] = E[3] = 0.0;
-      et[0] = et[1] = et[2] = 0.0;
-    }
-    double qc[4], pc[3];
-    qmul(E, q, qc);
-    qnormalize(qc);
-    for (int i = 0; i < 3; ++i) pc[i] = p[i] + et[i];
-    for (int m = 0; m < len; ++m) {
-      float* rec = poses + ((long long)sc * max_steps + lo + m) * kToolFields;
-      for (int i = 0; i < 3; ++i) rec[i] = float(pc[i]);
-      for (int i = 0; i < 4; ++i) rec[3 + i] = float(qc[i]);
-      for (int i = 0; i < 3; ++i) {
-        rec[7 + i] = float(pd[i]);
-        rec[10 + i] = float(om[i]);
-      }
-      for (int i = 0; i < 3; ++i) pc[i] += dt * pd[i];
-      double t4[4];
-      qmul(dq, qc, t4);
-      qnormalize(t4);
-      for (int i = 0; i < 4; ++i) qc[i] = t4[i];
-    }
-    // carry the pose after this chunk of actions
-    double DL[4], tL[3];
-    for (int i = 0; i < 4; ++i) DL[i] = __shfl_sync(0xffffffffu, D[i], 31);
-    for (int i = 0; i < 3; ++i) tL[i] = __shfl_sync(0xffffffffu, tr[i], 31);
-    double t4[4];
-    qmul(DL, q, t4);
-    qnormalize(t4);
-    for (int i = 0; i < 4; ++i) q[i] = t4[i];
-    for (int i = 0; i < 3; ++i) p[i] += tL[i];
+    __syncthreads();
   }
 }
 
 void launch_tool_forward(const Params& P, const float* pose0, const float* actions, int n_actions,
                          int spa, int n_steps, int max_steps, float* poses, cudaStream_t s) {
-  tool_forward_kernel<<<blocks_for((long long)P.S * 32, 128), 128, 0, s>>>(P.S, pose0, actions, n_actions, spa,
-                                                                         n_steps, max_steps, (double)P.dt, poses);
+  tool_forward_kernel<<<P.S, kToolThreads, 0, s>>>(P.S, pose0, actions, n_actions, spa, n_steps, max_steps,
+                                                   (double)P.dt, poses);
 }
 
 __device__ inline void qmulf(const float* a, const float* b, float* o) {
@@ -637,10 +639,13 @@ __device__ inline void rot_q_adjoint(const float* q, const float* gR, float* gq)
 
 // Reverse sweep of the kinematics: per-step tool gradients (p, R, pdot, omega)
 // -> action gradients (accumulated into action_grad, [S][n_actions][6]). One
-// warp per scene: the lanes evaluate every action's rotation increment and its
-// Jacobian (FP64) and stage the pose and gradient rows of 128 steps at a time
-// in shared memory; lane 0 walks the steps backwards in FP32 (the adjoint
-// recurrence of the orientation is serial).
+// CTA per scene: every action's rotation increment and its Jacobian (FP64) and
+// the pose and gradient rows of 128 steps at a time are staged in shared
+// memory. Only the orientation's adjoint recurrence is serial, so thread 0
+// walks nothing else (in FP32, the next step's operands loaded before this
+// step's stores); what a step needs before and gives after it is a thread per
+// step, and each action's sum a thread per component, last step first. Bound
+// by the latency of the walk (200 steps: 95 us with everything in it, 34 us so).
 constexpr int kToolChunk = 128;
 
 size_t tool_backward_smem(int n_actions) {
@@ -648,20 +653,21 @@ size_t tool_backward_smem(int n_actions) {
          sizeof(float);
 }
 
-__global__ void tool_backward_kernel(int S, const float* __restrict__ pose0,
-                                     const float* __restrict__ actions, int n_actions, int spa,
-                                     int n_steps, int max_steps, float dt,
-                                     const float* __restrict__ poses,
-                                     const float* __restrict__ tool_grad,
-                                     float* __restrict__ action_grad) {
+__global__ void __launch_bounds__(kToolThreads)
+tool_backward_kernel(const float* __restrict__ actions, int n_actions, int spa, int n_steps, int max_steps, float dt,
+                     const float* __restrict__ poses, const float* __restrict__ tool_grad,
+                     float* __restrict__ action_grad) {
   extern __shared__ float tsm[];
   float* sdq = tsm;                                  // [n_actions][16]: dq (4), d dq / d omega (12)
   float* sag = sdq + (size_t)n_actions * 16;         // [n_actions][6] action gradients
-  float* srec = sag + (size_t)n_actions * 6;         // [kToolChunk][13]
-  float* stg = srec + (size_t)kToolChunk * kToolFields;  // [kToolChunk][18]
-  const int sc = blockIdx.x, lane = threadIdx.x;
-  if (sc >= S) return;
-  for (int a = lane; a < n_actions; a += 32) {
+  // [kToolChunk][13]: the pose record; then 0-2 the position adjoint and 7-10
+  // the orientation adjoint that reach the step, 3-6 its unit quaternion q
+  float* srec = sag + (size_t)n_actions * 6;
+  // [kToolChunk][18]: the tool gradient; then 3-6 the rotation's share of the
+  // orientation adjoint, 7-10 qh, 11 1/|qq|, 12-17 the step's action gradient
+  float* stg = srec + (size_t)kToolChunk * kToolFields;
+  const int sc = blockIdx.x, tid = threadIdx.x;
+  for (int a = tid; a < n_actions; a += kToolThreads) {
     const float* act = actions + ((long long)sc * n_actions + a) * 6;
     double om[3] = {act[3], act[4], act[5]}, dqd[4], Jd[12];
     dq_of(om, (double)dt, dqd, Jd);
@@ -669,77 +675,119 @@ __global__ void tool_backward_kernel(int S, const float* __restrict__ pose0,
     for (int i = 0; i < 12; ++i) sdq[a * 16 + 4 + i] = float(Jd[i]);
     for (int i = 0; i < 6; ++i) sag[a * 6 + i] = 0.0f;
   }
-  float Pb[3] = {0, 0, 0}, Qb[4] = {0, 0, 0, 0};
+  float Pb[3] = {0, 0, 0}, Qb[4] = {0, 0, 0, 0};  // thread 0
   for (int n1 = n_steps; n1 > 0; n1 -= kToolChunk) {
     const int n0 = max(0, n1 - kToolChunk);
-    __syncwarp();
-    for (int i = lane; i < (n1 - n0) * kToolFields; i += 32)
+    __syncthreads();
+    for (int i = tid; i < (n1 - n0) * kToolFields; i += kToolThreads)
       srec[i] = poses[((long long)sc * max_steps + n0) * kToolFields + i];
-    for (int i = lane; i < (n1 - n0) * kToolGradFields; i += 32)
+    for (int i = tid; i < (n1 - n0) * kToolGradFields; i += kToolThreads)
       stg[i] = tool_grad[((long long)sc * max_steps + n0) * kToolGradFields + i];
-    __syncwarp();
-    if (lane == 0) {
-      for (int n = n1 - 1; n >= n0; --n) {
-        const float* rec = srec + (n - n0) * kToolFields;
+    __syncthreads();
+    for (int n = n0 + tid; n < n1; n += kToolThreads) {
+      float* rec = srec + (n - n0) * kToolFields;
+      float* tg = stg + (n - n0) * kToolGradFields;
+      // the stored pose (a unit quaternion to FP32 precision) is re-normalised
+      float q[4], qq[4], gq[4];
+      const float qr = rsqrtf(rec[3] * rec[3] + rec[4] * rec[4] + rec[5] * rec[5] + rec[6] * rec[6]);
+      for (int i = 0; i < 4; ++i) q[i] = rec[3 + i] * qr;
+      // q_{n+1} = qh = qq / |qq|, qq = dq q
+      qmulf(sdq + min(n / spa, n_actions - 1) * 16, q, qq);
+      const float inq = rsqrtf(qq[0] * qq[0] + qq[1] * qq[1] + qq[2] * qq[2] + qq[3] * qq[3]);
+      rot_q_adjoint(q, tg + 3, gq);
+      for (int i = 0; i < 4; ++i) {
+        rec[3 + i] = q[i];
+        tg[3 + i] = gq[i];
+        tg[7 + i] = qq[i] * inq;
+      }
+      tg[11] = inq;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      float g[12], dq[4];
+      auto load = [&](int n) {
         const float* tg = stg + (n - n0) * kToolGradFields;
-        const int a = min(n / spa, n_actions - 1);
-        const float* dq = sdq + a * 16;
-        const float* Jdq = dq + 4;
-        // the stored pose (a unit quaternion to FP32 precision) is re-normalised
-        float q[4];
-        const float qr = rsqrtf(rec[3] * rec[3] + rec[4] * rec[4] + rec[5] * rec[5] + rec[6] * rec[6]);
-        for (int i = 0; i < 4; ++i) q[i] = rec[3 + i] * qr;
+        const float* d = sdq + min(n / spa, n_actions - 1) * 16;
+#pragma unroll
+        for (int i = 0; i < 12; ++i) g[i] = tg[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) dq[i] = d[i];
+      };
+      load(n1 - 1);
+      for (int n = n1 - 1; n >= n0; --n) {
+        float* rec = srec + (n - n0) * kToolFields;
+        float h[12], e[4];
+#pragma unroll
+        for (int i = 0; i < 12; ++i) h[i] = g[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) e[i] = dq[i];
+        load(n > n0 ? n - 1 : n);
+        const float dotq = h[7] * Qb[0] + h[8] * Qb[1] + h[9] * Qb[2] + h[10] * Qb[3];
+        float r[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) r[i] = (Qb[i] - h[7 + i] * dotq) * h[11];
         // p_{n+1} = p_n + dt pdot_n
-        float pdb[3], pb[3];
+#pragma unroll
         for (int i = 0; i < 3; ++i) {
-          pdb[i] = tg[12 + i] + dt * Pb[i];
-          pb[i] = tg[i] + Pb[i];
+          rec[i] = Pb[i];
+          Pb[i] += h[i];
         }
-        // q_{n+1} = qq / |qq|, qq = dq q
-        float qq[4];
-        qmulf(dq, q, qq);
-        const float inq = rsqrtf(qq[0] * qq[0] + qq[1] * qq[1] + qq[2] * qq[2] + qq[3] * qq[3]);
-        const float qh[4] = {qq[0] * inq, qq[1] * inq, qq[2] * inq, qq[3] * inq};
-        const float dotq = qh[0] * Qb[0] + qh[1] * Qb[1] + qh[2] * Qb[2] + qh[3] * Qb[3];
-        float qqb[4];
-        for (int i = 0; i < 4; ++i) qqb[i] = (Qb[i] - qh[i] * dotq) * inq;
-        // qq = L(dq) q: qb = L(dq)^T qqb; dqb = Rm(q)^T qqb with qq = Rm(q) dq
-        float qb[4], dqb[4];
-        qb[0] = dq[0] * qqb[0] + dq[1] * qqb[1] + dq[2] * qqb[2] + dq[3] * qqb[3];
-        qb[1] = -dq[1] * qqb[0] + dq[0] * qqb[1] + dq[3] * qqb[2] - dq[2] * qqb[3];
-        qb[2] = -dq[2] * qqb[0] - dq[3] * qqb[1] + dq[0] * qqb[2] + dq[1] * qqb[3];
-        qb[3] = -dq[3] * qqb[0] + dq[2] * qqb[1] - dq[1] * qqb[2] + dq[0] * qqb[3];
-        dqb[0] = q[0] * qqb[0] + q[1] * qqb[1] + q[2] * qqb[2] + q[3] * qqb[3];
-        dqb[1] = -q[1] * qqb[0] + q[0] * qqb[1] - q[3] * qqb[2] + q[2] * qqb[3];
-        dqb[2] = -q[2] * qqb[0] + q[3] * qqb[1] + q[0] * qqb[2] - q[1] * qqb[3];
-        dqb[3] = -q[3] * qqb[0] - q[2] * qqb[1] + q[1] * qqb[2] + q[0] * qqb[3];
-        float gq[4];
-        rot_q_adjoint(q, tg + 3, gq);
-        for (int i = 0; i < 4; ++i) qb[i] += gq[i];
-        float* ag = sag + a * 6;
-        for (int k = 0; k < 3; ++k) {
-          float omb = tg[15 + k];
-          for (int i = 0; i < 4; ++i) omb += Jdq[3 * i + k] * dqb[i];
-          ag[k] += pdb[k];
-          ag[3 + k] += omb;
-        }
-        for (int i = 0; i < 3; ++i) Pb[i] = pb[i];
-        for (int i = 0; i < 4; ++i) Qb[i] = qb[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) rec[7 + i] = Qb[i];
+        // qq = L(dq) q: qb = L(dq)^T qqb
+        Qb[0] = e[0] * r[0] + e[1] * r[1] + e[2] * r[2] + e[3] * r[3] + h[3];
+        Qb[1] = -e[1] * r[0] + e[0] * r[1] + e[3] * r[2] - e[2] * r[3] + h[4];
+        Qb[2] = -e[2] * r[0] - e[3] * r[1] + e[0] * r[2] + e[1] * r[3] + h[5];
+        Qb[3] = -e[3] * r[0] + e[2] * r[1] - e[1] * r[2] + e[0] * r[3] + h[6];
       }
     }
+    __syncthreads();
+    for (int n = n0 + tid; n < n1; n += kToolThreads) {
+      const float* rec = srec + (n - n0) * kToolFields;
+      float* tg = stg + (n - n0) * kToolGradFields;
+      const float* q = rec + 3;
+      const float* Qn = rec + 7;
+      const float* qh = tg + 7;
+      const float* Jdq = sdq + min(n / spa, n_actions - 1) * 16 + 4;
+      const float dotq = qh[0] * Qn[0] + qh[1] * Qn[1] + qh[2] * Qn[2] + qh[3] * Qn[3];
+      float r[4], dqb[4];
+      for (int i = 0; i < 4; ++i) r[i] = (Qn[i] - qh[i] * dotq) * tg[11];
+      // dqb = Rm(q)^T qqb with qq = Rm(q) dq
+      dqb[0] = q[0] * r[0] + q[1] * r[1] + q[2] * r[2] + q[3] * r[3];
+      dqb[1] = -q[1] * r[0] + q[0] * r[1] - q[3] * r[2] + q[2] * r[3];
+      dqb[2] = -q[2] * r[0] + q[3] * r[1] + q[0] * r[2] - q[1] * r[3];
+      dqb[3] = -q[3] * r[0] - q[2] * r[1] + q[1] * r[2] + q[0] * r[3];
+      for (int k = 0; k < 3; ++k) {
+        float omb = tg[15 + k];
+        for (int i = 0; i < 4; ++i) omb += Jdq[3 * i + k] * dqb[i];
+        tg[12 + k] += dt * rec[k];
+        tg[15 + k] = omb;
+      }
+    }
+    __syncthreads();
+    const int a0 = min(n0 / spa, n_actions - 1), a1 = min((n1 - 1) / spa, n_actions - 1);
+    for (int t = tid; t < (a1 - a0 + 1) * 6; t += kToolThreads) {
+      const int a = a0 + t / 6, k = t % 6;
+      const long long lo = max((long long)a * spa, (long long)n0);
+      const long long hi = a == n_actions - 1 ? n1 : min((long long)(a + 1) * spa, (long long)n1);
+      float v = sag[a * 6 + k];
+#pragma unroll 4
+      for (long long n = hi - 1; n >= lo; --n) v += stg[(n - n0) * kToolGradFields + 12 + k];
+      sag[a * 6 + k] = v;
+    }
   }
-  __syncwarp();
-  for (int i = lane; i < n_actions * 6; i += 32) action_grad[(long long)sc * n_actions * 6 + i] += sag[i];
+  __syncthreads();
+  for (int i = tid; i < n_actions * 6; i += kToolThreads) action_grad[(long long)sc * n_actions * 6 + i] += sag[i];
 }
 
-void launch_tool_backward(const Params& P, const float* pose0, const float* actions, int n_actions,
+void launch_tool_backward(const Params& P, const float* actions, int n_actions,
                           int spa, int n_steps, int max_steps, const float* poses,
                           const float* tool_grad, float* action_grad, cudaStream_t s) {
   const size_t smem = tool_backward_smem(n_actions);
   if (smem > 48 * 1024) cudaFuncSetAttribute(tool_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(smem));
-  tool_backward_kernel<<<P.S, 32, smem, s>>>(P.S, pose0, actions, n_actions, spa, n_steps, max_steps, P.dt, poses,
-                                            tool_grad, action_grad);
+  tool_backward_kernel<<<P.S, kToolThreads, smem, s>>>(actions, n_actions, spa, n_steps, max_steps, P.dt, poses,
+                                                       tool_grad, action_grad);
 }
 
 // ---------------------------------------------------------------------------

@@ -121,7 +121,7 @@ void launch_gather_rows(const float* src, float* dst, const int* pid, int N, int
 // tool kinematics
 void launch_tool_forward(const Params& P, const float* pose0, const float* actions, int n_actions,
                          int spa, int n_steps, int max_steps, float* poses, cudaStream_t s);
-void launch_tool_backward(const Params& P, const float* pose0, const float* actions, int n_actions,
+void launch_tool_backward(const Params& P, const float* actions, int n_actions,
                           int spa, int n_steps, int max_steps, const float* poses,
                           const float* tool_grad, float* action_grad, cudaStream_t s);
 

@@ -529,6 +529,9 @@ void set_params(sim_h h) {
   P.eps_c = c.contact_eps;
   P.inv_ell = c.contact_soft > 0.0f ? 1.0f / c.contact_soft : float(c.grid_n);
   P.mu_f = c.friction;
+  const double reach = std::sqrt((double)P.half[0] * P.half[0] + (double)P.half[1] * P.half[1] +
+                                 (double)P.half[2] * P.half[2]) + std::max(P.eps_c, 0.0f);
+  P.reach2 = float(reach * reach * 1.001 + 1e-12);
 }
 
 // Run chunk c (steps [c k, min(T, c k + k))) from its checkpoint into chunk
@@ -1654,7 +1657,7 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
       cudaMemsetAsync(h->action_grad, 0, sizeof(float) * h->S * h->n_actions * 6, s);
       {
         Prof pr(h, "tool_adj", s);
-        launch_tool_backward(P, h->pose0, h->actions, h->n_actions, h->spa, T, h->max_steps, h->poses,
+        launch_tool_backward(P, h->actions, h->n_actions, h->spa, T, h->max_steps, h->poses,
                              h->tool_grad, h->action_grad, s);
       }
       h->launches += 1;

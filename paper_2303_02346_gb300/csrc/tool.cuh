@@ -41,6 +41,15 @@ __device__ inline void load_tool(const float* pose, ToolState& t) {
   quat_rot(t.q, t.R);
 }
 
+// Whether a node is so far from the tool's centre that contact cannot act
+// there (phi >= |x - p| - |half| >= eps_c; a NaN pose never acts either). Most
+// nodes are: they need three words of the pose and no rotation (64 scenes on
+// 64^3 grids: grid adjoint 38.9 -> 32.7 us, grid update 24.6 -> 22.9 us).
+__device__ inline bool tool_far(const Params& P, const float* pose, const float* xi) {
+  const float d0 = xi[0] - pose[0], d1 = xi[1] - pose[1], d2 = xi[2] - pose[2];
+  return !(d0 * d0 + d1 * d1 + d2 * d2 <= P.reach2);
+}
+
 // Box SDF in the tool frame: phi and its gradient g (unit) w.r.t. y.
 struct SdfEval {
   float r[3], y[3], sgn[3], e[3];
