@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "mpm_gas.h"
+#include "sum2.cuh"
 #include "sur_ptx.cuh"
 
 namespace {
@@ -172,19 +173,8 @@ advect_kernel(Geo g, const float4* __restrict__ pk, const uint8_t* __restrict__ 
   dn[c] = v.w;
 }
 
-// Sum of a thread's values to about 48 bits in two FP32 words (Knuth's
-// two-sum): FP64 adds for every cell bound the two kernels below (GB300's FP64
-// rate is a small fraction of its FP32 rate), so FP64 is left to one value a
-// thread.
-struct Sum2 {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float v) {
-    const float s = __fadd_rn(hi, v), bb = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(v, bb)));
-    hi = s;
-  }
-  __device__ __forceinline__ double value() const { return double(hi) + double(lo); }
-};
+// FP64 adds for every cell would bound the two kernels below (GB300's FP64
+// rate is a small fraction of its FP32 rate): a thread sums in two FP32 words.
 constexpr int kSumPlanes = 16;  // planes along i a thread walks through
 
 // b = divergence of un on fluid cells (solid neighbours hold zero velocity);

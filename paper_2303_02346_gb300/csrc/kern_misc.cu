@@ -7,6 +7,7 @@
 #include "kernels.h"
 #include "perm.h"
 #include "share.h"
+#include "sum2.cuh"
 
 namespace mpm {
 
@@ -809,36 +810,90 @@ __device__ inline void block_add_double(double v, double* out) {
 }
 
 // L_s = w sum |x - t|^2 over particles of scene `scene` (-1: all, per-scene
-// totals into loss[scene]); adj_x += 2 w (x - t).
-__global__ void position_loss_kernel(Params P, const float* __restrict__ st, const uint32_t* __restrict__ tag,
-                                     int scene, float tx, float ty, float tz, float w,
-                                     float* __restrict__ adj, double* __restrict__ loss) {
+// totals into loss[scene]); adj_x += 2 w (x - t). The FP64 units would bound it
+// (98 us at 2M particles with the sum in FP64 throughout, 21 us so), so a thread
+// sums the exact squares of its kLossItems particles in two FP32 words, as far
+// as FP32 holds them, and goes to FP64 once; particles are sorted by scene, so
+// its particles seldom belong to more than one loss entry, nor do a CTA's.
+constexpr int kLossItems = 8;
+
+__global__ void __launch_bounds__(256)
+position_loss_kernel(Params P, const float* __restrict__ st, const uint32_t* __restrict__ tag,
+                     int scene, float tx, float ty, float tz, float w,
+                     float* __restrict__ adj, double* __restrict__ loss) {
+  __shared__ double ws[8];
+  __shared__ int wt[8];
   const int N = P.N;
-  int p = blockIdx.x * blockDim.x + threadIdx.x;
-  double l = 0.0;
-  int sc = -1;
-  if (p < N) {
-    sc = tag_scene(tag[p]);
-    if (scene < 0 || sc == scene) {
-      float d0 = st[p] - tx, d1 = st[N + p] - ty, d2 = st[2 * N + p] - tz;
-      l = (double)w * ((double)d0 * d0 + (double)d1 * d1 + (double)d2 * d2);
-      adj[p] += 2.0f * w * d0;
-      adj[N + p] += 2.0f * w * d1;
-      adj[2 * N + p] += 2.0f * w * d2;
+  const int base = blockIdx.x * (256 * kLossItems) + threadIdx.x;
+  int cur = -1;
+  Sum2 acc;
+#pragma unroll
+  for (int it = 0; it < kLossItems; it += 4) {
+    uint32_t tg[4];
+    float d[4][3], g[4][3];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {  // all loads first; past the end: the last particle, not used
+      const int p = min(base + (it + u) * 256, N - 1);
+      tg[u] = tag[p];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        d[u][k] = st[k * N + p];
+        g[u][k] = adj[k * N + p];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int p = base + (it + u) * 256, sc = tag_scene(tg[u]);
+      if (p >= N || (scene >= 0 && sc != scene)) continue;
+      const float d0 = d[u][0] - tx, d1 = d[u][1] - ty, d2 = d[u][2] - tz;
+      adj[p] = g[u][0] + 2.0f * w * d0;
+      adj[N + p] = g[u][1] + 2.0f * w * d1;
+      adj[2 * N + p] = g[u][2] + 2.0f * w * d2;
+      const int t = scene < 0 ? sc : 0;
+      if (t != cur) {
+        if (cur >= 0) atomicAdd(loss + cur, (double)w * acc.value());
+        acc = Sum2();
+        cur = t;
+      }
+      if (d0 * d0 + d1 * d1 + d2 * d2 < 1e30f) {
+        acc.add_square(d0);
+        acc.add_square(d1);
+        acc.add_square(d2);
+      } else {  // a target far outside, or NaN
+        atomicAdd(loss + t, (double)w * ((double)d0 * d0 + (double)d1 * d1 + (double)d2 * d2));
+      }
     }
   }
-  // one atomic per warp when its particles share the loss entry (particles are
-  // sorted by scene, so only warps at a scene boundary add lane by lane)
-  const int t = (p < N && (scene < 0 || sc == scene)) ? (scene < 0 ? sc : 0) : -1;
-  const int tmax = __reduce_max_sync(0xffffffffu, t);
-  const int tmin = __reduce_min_sync(0xffffffffu, t >= 0 ? t : INT_MAX);
-  if (tmax < 0) return;
-  if (tmin == tmax) {
+  double l = cur >= 0 ? (double)w * acc.value() : 0.0;
+  // one atomic per CTA when its particles share the loss entry
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int tmax = __reduce_max_sync(0xffffffffu, cur);
+  const int tmin = __reduce_min_sync(0xffffffffu, cur >= 0 ? cur : INT_MAX);
+  const bool one = tmax >= 0 && tmin == tmax;
+  if (one) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0 && l != 0.0) atomicAdd(loss + tmax, l);
-  } else if (l != 0.0) {
-    atomicAdd(loss + t, l);
+  } else if (cur >= 0) {
+    atomicAdd(loss + cur, l);
+  }
+  if (lane == 0) {
+    ws[wid] = l;
+    wt[wid] = one ? tmax : -1;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int t = -1;
+    double s = 0.0;
+    for (int i = 0; i < 8; ++i) {
+      if (wt[i] < 0) continue;
+      if (wt[i] != t && t >= 0) {
+        atomicAdd(loss + t, s);
+        s = 0.0;
+      }
+      t = wt[i];
+      s += ws[i];
+    }
+    if (t >= 0) atomicAdd(loss + t, s);
   }
 }
 
@@ -846,7 +901,7 @@ void launch_position_loss(const Params& P, const float* st, const uint32_t* tag,
                           float tx, float ty, float tz, float w, float* adj, double* loss,
                           cudaStream_t s) {
   if (P.N == 0) return;
-  position_loss_kernel<<<blocks_for(P.N, 256), 256, 0, s>>>(P, st, tag, scene, tx, ty, tz, w, adj, loss);
+  position_loss_kernel<<<blocks_for(P.N, 256 * kLossItems), 256, 0, s>>>(P, st, tag, scene, tx, ty, tz, w, adj, loss);
 }
 
 // P2G mass of the particles of one scene into a dense float grid
@@ -875,18 +930,26 @@ void launch_mass_scatter(const Params& P, const float* st, const uint32_t* tag, 
   mass_scatter_kernel<<<blocks_for(P.N, 256), 256, 0, s>>>(P, st, tag, scene, mgrid);
 }
 
-// L = sum (m - m*)^2 / M^2 + sum m d* / M; dL/dm per node
+// L = sum (m - m*)^2 / M^2 + sum m d* / M; dL/dm per node, in FP64. Most nodes
+// hold no mass and want none: they add nothing, and their dL/dm is one rounded
+// product of two FP32 numbers, the same in FP32. FP64, whose units bound the
+// rest, is left to the others (128^3 nodes: 83 -> 9 us).
 __global__ void mass_loss_nodes_kernel(long long n3, const float* __restrict__ mg, const float* __restrict__ tm,
                                        const float* __restrict__ td, float inv_M, float* __restrict__ dLdm,
                                        double* __restrict__ loss) {
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   double l = 0.0;
   if (i < n3) {
-    double m = mg[i], d = m - (double)tm[i];
-    l = d * d * (double)inv_M * inv_M + m * (double)td[i] * inv_M;
-    dLdm[i] = float(2.0 * d * inv_M * inv_M + (double)td[i] * inv_M);
+    const float mf = mg[i], tf = tm[i], df = td[i], g = df * inv_M;
+    if (mf == 0.0f && tf == 0.0f && isfinite(g)) {
+      dLdm[i] = g;
+    } else {
+      double m = mf, d = m - (double)tf;
+      l = d * d * (double)inv_M * inv_M + m * (double)df * inv_M;
+      dLdm[i] = float(2.0 * d * inv_M * inv_M + (double)df * inv_M);
+    }
   }
-  block_add_double(l, loss);
+  if (__syncthreads_or(l != 0.0)) block_add_double(l, loss);
 }
 
 void launch_mass_loss_nodes(long long n3, const float* mgrid, const float* tm, const float* td,
