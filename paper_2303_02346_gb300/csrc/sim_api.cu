@@ -378,7 +378,7 @@ void do_sort(sim_h h, const float* st_in, const uint32_t* tag_in, const int* pid
              uint32_t* tag_out, int* pid_out, cudaStream_t s) {
   Prof pr(h, "sort", s);
   launch_sort(h->P, st_in, tag_in, pid_in, st_out, tag_out, pid_out, h->sb, s);
-  h->launches += h->P.N > 0 ? 6 : 0;
+  h->launches += h->P.N > 0 ? 7 : 0;
 }
 
 // Wait for the stream and read the error word. The word is copied to pinned
