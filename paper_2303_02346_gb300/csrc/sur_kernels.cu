@@ -80,7 +80,10 @@ __device__ __forceinline__ bool make_stencil(const float* x, int n, Stencil& s) 
   for (int d = 0; d < 3; ++d) {
     const float xs = x[d] * n;
     const int b = static_cast<int>(floorf(xs - 0.5f));
-    const float f = xs - b;
+    // one rounding, of f itself: x n rounded first would leave an error of its
+    // own size in f wherever n is not a power of two (adjoint at n = 45: 1.4e-6
+    // against 1.3e-7), and whether the compiler fuses the two is its own choice
+    const float f = __fmaf_rn(x[d], static_cast<float>(n), -static_cast<float>(b));
     s.base[d] = b;
     s.fx[d] = f;
     s.w[0][d] = 0.5f * (1.5f - f) * (1.5f - f);
