@@ -752,7 +752,7 @@ void sweep(const Geo& g, const float* p_in, float* p_out, const float* rhs, cons
 // The projection's sweeps from p = 0, in pairs from the size on where those are
 // faster (figures at jacobi2_kernel); returns the buffer that holds the result and adds the
 // launches.
-constexpr int kPairFrom = 160;
+constexpr int kPairFrom = 160, kMaxGrid = 512;
 PairShape pair_shape(int n, int sms) {
   PairShape q;
   q.tx = n / 4;
@@ -768,6 +768,14 @@ PairShape pair_shape(int n, int sms) {
   q.grid_i = (n + q.seg - 1) / q.seg;
   q.smem = sizeof(float4) * ((size_t)3 * q.rows * q.tx + kStages * pair_stage_f4(q.tx, q.rows));
   return q;
+}
+
+// The largest need of any grid size. The limit belongs to the function, not to a
+// handle: one set to a handle's own need would be lowered by the next, smaller one.
+int pair_smem_limit(int sms) {
+  size_t most = 0;
+  for (int n = kPairFrom; n <= kMaxGrid; n += 4) most = std::max(most, pair_shape(n, sms).smem);
+  return int(most);
 }
 
 float* sweeps(gas_h h, const float* rhs, const float* mean, cudaStream_t st, long long* launches) {
@@ -889,7 +897,7 @@ extern "C" {
 sim_status gas_create(const gas_config* cfg, const uint8_t* solid, gas_h* out) {
   if (!cfg || !solid || !out) return SIM_E_ARG;
   *out = nullptr;
-  if (cfg->n < 8 || cfg->n > 512 || !(cfg->dt > 0.0f) || cfg->jacobi_iters < 1 || cfg->max_steps < 1) return SIM_E_ARG;
+  if (cfg->n < 8 || cfg->n > kMaxGrid || !(cfg->dt > 0.0f) || cfg->jacobi_iters < 1 || cfg->max_steps < 1) return SIM_E_ARG;
   gas_h h = new mpm_gas();
   h->cfg = *cfg;
   const int n = cfg->n;
@@ -918,7 +926,7 @@ sim_status gas_create(const gas_config* cfg, const uint8_t* solid, gas_h* out) {
   ok = ok && cudaMalloc(&h->err, sizeof(int)) == cudaSuccess && cudaMemset(h->err, 0, sizeof(int)) == cudaSuccess;
   if (ok && n % 4 == 0 && n >= kPairFrom)
     ok = cudaFuncSetAttribute(jacobi2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(pair_shape(n, h->sms).smem)) == cudaSuccess;
+                              pair_smem_limit(h->sms)) == cudaSuccess;
   ok = ok && cudaMemcpy(h->solid, solid, n3, cudaMemcpyHostToDevice) == cudaSuccess;
   if (ok) {
     neighbours_kernel<<<cell_grid(n), kCellBlock>>>(n, h->solid, h->nbr);
