@@ -21,6 +21,7 @@
 #include <utility>
 #include <vector>
 
+#include "graph.h"
 #include "mpm_gas.h"
 #include "sum2.cuh"
 #include "sur_ptx.cuh"
@@ -852,15 +853,12 @@ long long enqueue_backward(gas_h h, int s, cudaStream_t st) {
 sim_status run_graph(gas_h h, std::vector<cudaGraphExec_t>& cache, std::vector<long long>& counts, int s,
                      long long (*enq)(gas_h, int, cudaStream_t)) {
   if (!cache[s]) {
-    cudaGraph_t graph;
-    cudaError_t e = cudaStreamBeginCapture(h->cstream, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) return gcuda(h, e, "gas graph capture");
-    counts[s] = enq(h, s, h->cstream);
-    e = cudaStreamEndCapture(h->cstream, &graph);
-    if (e != cudaSuccess) return gcuda(h, e, "gas graph capture");
-    e = cudaGraphInstantiate(&cache[s], graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) return gcuda(h, e, "gas graph instantiate");
+    const cudaError_t e =
+        mpm::capture_graph(h->cstream, 0, [&](cudaStream_t cs) { counts[s] = enq(h, s, cs); }, &cache[s]);
+    if (e != cudaSuccess) {
+      cudaGetLastError();  // reported here
+      return gcuda(h, e, "gas graph capture");
+    }
   }
   cudaError_t e = cudaGraphLaunch(cache[s], h->stream);
   if (e != cudaSuccess) return gcuda(h, e, "gas graph launch");

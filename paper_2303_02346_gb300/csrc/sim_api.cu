@@ -31,6 +31,7 @@
 #include <string>
 #include <vector>
 
+#include "graph.h"
 #include "kernels.h"
 #include "perm.h"
 #include "rigid.h"
@@ -795,27 +796,11 @@ cudaGraphExec_t capture(sim_h h, Fn fn, bool node_priority = false) {
     cudaGetLastError();
     return nullptr;
   }
-  if (cudaStreamBeginCapture(h->cstream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  fn(h->cstream);
-  cudaGraph_t graph = nullptr;
-  cudaError_t e = cudaStreamEndCapture(h->cstream, &graph);
-  if (e != cudaSuccess || !graph) {
-    cudaGetLastError();
-    return nullptr;
-  }
   cudaGraphExec_t exec = nullptr;
   // node_priority: kernels keep the priority of the stream they were captured
   // on (the backward's sweep and recompute streams) instead of taking the
   // launch stream's
-  e = cudaGraphInstantiate(&exec, graph, node_priority ? cudaGraphInstantiateFlagUseNodePriority : 0);
-  cudaGraphDestroy(graph);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
+  capture_graph(h->cstream, node_priority ? cudaGraphInstantiateFlagUseNodePriority : 0, fn, &exec);
   return exec;
 }
 
