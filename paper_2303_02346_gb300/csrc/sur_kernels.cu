@@ -504,9 +504,10 @@ __global__ void __launch_bounds__(kLbThreads) lift_bwd_kernel(SurGeom g, int bat
                                                               const float* __restrict__ wl,
                                                               const float* __restrict__ g_pred, float* grad_wl,
                                                               float* grad_bl, float* g_frames) {
-  __shared__ float sw[256];
+  __shared__ float4 sw4[64];  // read 16 bytes at a time
   __shared__ uint32_t rows[kLbThreads * kRowWords];
   __shared__ float4 sf[kLbThreads * 2];
+  float* sw = reinterpret_cast<float*>(sw4);
   for (int i = threadIdx.x; i < 256; i += blockDim.x) sw[i] = rbf(wl[i]);
   __syncthreads();
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -534,8 +535,7 @@ __global__ void __launch_bounds__(kLbThreads) lift_bwd_kernel(SurGeom g, int bat
           unpack8(raw[c], gv);
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
-            const float4 wa = reinterpret_cast<const float4*>(sw)[(c * 8 + e) * 2],
-                         wb = reinterpret_cast<const float4*>(sw)[(c * 8 + e) * 2 + 1];
+            const float4 wa = sw4[(c * 8 + e) * 2], wb = sw4[(c * 8 + e) * 2 + 1];
             const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
             for (int q = 0; q < 8; ++q) gf[q] += w[q] * gv[e];
