@@ -177,7 +177,8 @@ int sim_current_step(sim_h h);
  * The states the trajectory keeps are readable: step = -1 or the current step,
  * step 0 (the initial state) and, with checkpointing, every checkpoint step
  * c*checkpoint_every before the current step (App. A: one state per caching
- * step). Any other step: SIM_E_STATE. */
+ * step). Any other step: SIM_E_STATE. Device outputs are written after the work
+ * that is already on the legacy default stream. */
 sim_status sim_get_state(sim_h h, int scene, int step, float* x, float* v, float* C,
                          float* F, int on_device);
 

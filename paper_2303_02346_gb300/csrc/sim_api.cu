@@ -110,6 +110,7 @@ struct mpm_sim {
   cudaStream_t hstream = nullptr;  // highest priority: the reverse sweep while rstream recomputes
   cudaEvent_t ev_start = nullptr, ev_rec[kMaxBuffers] = {}, ev_adj[kMaxBuffers] = {};
   cudaEvent_t ev_join = nullptr;
+  cudaEvent_t ev_read = nullptr;  // sim_get_state's wait for the default stream
   float* adj = nullptr;
   float4 *gadj_v = nullptr, *gadj_m = nullptr;
   float* rows = nullptr;  // N x 24 caller-layout staging
@@ -921,6 +922,7 @@ sim_status sim_destroy(sim_h h) {
   }
   if (h->ev_start) cudaEventDestroy(h->ev_start);
   if (h->ev_join) cudaEventDestroy(h->ev_join);
+  if (h->ev_read) cudaEventDestroy(h->ev_read);
   if (h->rstream) cudaStreamDestroy(h->rstream);
   if (h->hstream) cudaStreamDestroy(h->hstream);
   if (h->words) cudaFreeHost(h->words);
@@ -1323,11 +1325,20 @@ sim_status sim_get_state(sim_h h, int scene, int step, float* x, float* v, float
       off += (size_t)nc[q] * cnt;
     }
   }
+  cudaError_t e = cudaSuccess;
+  if (on_device && h->stream) {
+    // the caller's buffers may still be in use by work on the default stream
+    // (a buffer that an allocator handed on): write after it
+    if (!h->ev_read) e = cudaEventCreateWithFlags(&h->ev_read, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(h->ev_read, cudaStreamLegacy);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, h->ev_read, 0);
+    if (e != cudaSuccess) return cuda_fail(h, e, "sim_get_state");
+  }
   if (x || v || C || F) {
     launch_read_state(h->P, src, h->tag0, pid, lo, cnt, dev[0], dev[1], dev[2], dev[3], h->stream);
     h->launches += N > 0 && cnt > 0 ? 1 : 0;
   }
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   for (int q = 0; q < 4 && !on_device && e == cudaSuccess; ++q)
     if (host[q] && cnt)
       e = cudaMemcpyAsync(host[q], dev[q], sizeof(float) * nc[q] * cnt, cudaMemcpyDeviceToHost, h->stream);

@@ -42,6 +42,7 @@ class Simulator:
             contact_eps=scene.contact_eps, contact_soft=scene.contact_soft,
             friction=scene.friction, cuda_stream=stream, resort_every=resort_every,
             no_graphs=not graphs)
+        self.stream = int(stream)
         self.k = k
         self.max_steps = T
         self.N = int(scene.n_particles)
@@ -77,6 +78,16 @@ class Simulator:
         if self.scene.tool_enabled:
             self.set_tool()
 
+    def _empty(self, *shape):
+        """An output buffer of this shape. The library writes it on the handle's stream, but the allocator
+        orders its reuse by the current one, where work on the block's last owner may be pending: the
+        handle's stream waits for that. (The calls that fill outputs return when they are written.)"""
+        out = torch.empty(*shape, dtype=torch.float32, device=self.device)
+        current = torch.cuda.current_stream(self.device)
+        if current.cuda_stream != self.stream:
+            torch.cuda.ExternalStream(self.stream, device=self.device).wait_stream(current)
+        return out
+
     # -- stepping and state -------------------------------------------------
     def step(self, n):
         B.sim_step(self.h, n)
@@ -87,12 +98,10 @@ class Simulator:
 
     def state(self, scene=-1, with_CF=False, step=-1):
         cnt = self.N if scene < 0 else int(self.scene.scene_counts[scene])
-        x = torch.empty(cnt, 3, dtype=torch.float32, device=self.device)
-        v = torch.empty(cnt, 3, dtype=torch.float32, device=self.device)
+        x, v = self._empty(cnt, 3), self._empty(cnt, 3)
         C = F = None
         if with_CF:
-            C = torch.empty(cnt, 3, 3, dtype=torch.float32, device=self.device)
-            F = torch.empty(cnt, 3, 3, dtype=torch.float32, device=self.device)
+            C, F = self._empty(cnt, 3, 3), self._empty(cnt, 3, 3)
         B.sim_get_state(self.h, scene, step, x, v, C, F)
         return (x, v, C, F) if with_CF else (x, v)
 
@@ -113,7 +122,7 @@ class Simulator:
         dev = self.device
         e = torch.as_tensor(ell, dtype=torch.float32, device=dev).contiguous()
         gg = torch.as_tensor(g, dtype=torch.float32, device=dev).reshape(-1, 3).contiguous()
-        out = torch.empty_like(gg)
+        out = self._empty(*gg.shape)
         B.sim_share_gradients(self.h, scene, e, radius, tau, gg, out)
         return out
 
@@ -128,18 +137,17 @@ class Simulator:
     def tool_pose(self, step, scene=-1):
         """(S or 1, 13) tool pose at the start of `step`: position, quaternion
         (w, x, y, z), linear and angular velocity."""
-        out = torch.empty(self.S if scene < 0 else 1, 13, dtype=torch.float32, device=self.device)
+        out = self._empty(self.S if scene < 0 else 1, 13)
         B.sim_get_tool_pose(self.h, scene, step, out)
         return out
 
     def backward(self, want_actions=True):
-        gx = torch.empty(self.N, 3, dtype=torch.float32, device=self.device)
-        gv = torch.empty(self.N, 3, dtype=torch.float32, device=self.device)
+        gx, gv = self._empty(self.N, 3), self._empty(self.N, 3)
         ga = None
         if want_actions and self.scene.tool_enabled:
             n_max = -(-self.max_steps // max(int(self.scene.substeps_per_action), 1))
             n_act = min(self.scene.tool_actions.shape[-2], n_max)
-            ga = torch.empty(self.S, n_act, 6, dtype=torch.float32, device=self.device)
+            ga = self._empty(self.S, n_act, 6)
         B.sim_backward(self.h, gx, gv, ga)
         return gx, gv, ga
 
