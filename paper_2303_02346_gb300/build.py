@@ -56,7 +56,7 @@ KERNEL_SOURCES = {
     "mpm_adj": ["common.cuh", "constitutive.cuh", "scatter.cuh", "tool.cuh", "kernels.h", "kern_adj.cu"],
     "surrogate": ["sur_ptx.cuh", "sur_kernels.h", "sur_conv.cu", "sur_wgrad.cu", "sur_kernels.cu"],
     "share": ["common.cuh", "kernels.h", "share.h", "kern_share.cu"],
-    "gas": ["sum2.cuh", "sur_ptx.cuh", "gas.cu"],
+    "gas": ["sum3.cuh", "sur_ptx.cuh", "gas.cu"],
     "rigid": ["common.cuh", "constitutive.cuh", "rigid.h", "kern_rigid.cu"],
 }
 

@@ -7,7 +7,7 @@
 #include "kernels.h"
 #include "perm.h"
 #include "share.h"
-#include "sum2.cuh"
+#include "sum3.cuh"
 
 namespace mpm {
 
@@ -846,9 +846,9 @@ __device__ inline void block_add_double(double v, double* out) {
 // L_s = w sum |x - t|^2 over particles of scene `scene` (-1: all, per-scene
 // totals into loss[scene]); adj_x += 2 w (x - t). The FP64 units would bound it
 // (98 us at 2M particles with the sum in FP64 throughout, 17 us so), so a thread
-// sums the exact squares of its kLossItems particles in two FP32 words, as far
-// as FP32 holds them, and goes to FP64 once; particles are sorted by scene, so
-// its particles seldom belong to more than one loss entry, nor do a CTA's.
+// sums the exact squares of its kLossItems particles in three FP32 words, which
+// loses nothing against FP64, and goes to FP64 once; particles are sorted by scene,
+// so its particles seldom belong to more than one loss entry, nor do a CTA's.
 constexpr int kLossItems = 8;
 
 __global__ void __launch_bounds__(256)
@@ -860,7 +860,7 @@ position_loss_kernel(Params P, const float* __restrict__ st, const uint32_t* __r
   const int N = P.N;
   const int base = blockIdx.x * (256 * kLossItems) + threadIdx.x;
   int cur = -1;
-  Sum2 acc;
+  Sum3 acc;
 #pragma unroll
   for (int it = 0; it < kLossItems; it += 4) {
     uint32_t tg[4];
@@ -886,14 +886,15 @@ position_loss_kernel(Params P, const float* __restrict__ st, const uint32_t* __r
       const int t = scene < 0 ? sc : 0;
       if (t != cur) {
         if (cur >= 0) atomicAdd(loss + cur, (double)w * acc.value());
-        acc = Sum2();
+        acc = Sum3();
         cur = t;
       }
-      if (d0 * d0 + d1 * d1 + d2 * d2 < 1e30f) {
+      const float sq = d0 * d0 + d1 * d1 + d2 * d2;
+      if (sq > 1e-25f && sq < 1e30f) {
         acc.add_square(d0);
         acc.add_square(d1);
         acc.add_square(d2);
-      } else {  // a target far outside, or NaN
+      } else if (sq != 0.0f || d0 != 0.0f || d1 != 0.0f || d2 != 0.0f) {  // a target far outside, one met to 3e-13, or NaN
         atomicAdd(loss + t, (double)w * ((double)d0 * d0 + (double)d1 * d1 + (double)d2 * d2));
       }
     }
