@@ -324,7 +324,7 @@ constexpr int kRowWords = 17;  // words per node of a transposed channel row (16
 // transpose in its own shared memory: each lane leaves its node's 32 channels
 // there and takes one channel of all 32 nodes, so that a lane accumulates 3
 // entries instead of 96 (which took 255 registers and spills); no barrier.
-// The weights are read 16 bytes at a time. 8 frames of 64^3: training 164 -> 102
+// The weights are read 16 bytes at a time. 8 frames of 64^3: training 170 -> 99
 // us, inference 67 -> 46.
 template <int MODE>
 __global__ void __launch_bounds__(kProjThreads, (MODE & 2) ? 2 : (MODE & 4) ? 3 : 4) proj_kernel(SurGeom g, int batch,
@@ -443,15 +443,34 @@ __global__ void __launch_bounds__(kProjThreads, (MODE & 2) ? 2 : (MODE & 4) ? 3 
       __syncwarp();
       const uint32_t* col = rows + warp * 32 * kRowWords + lane / 2;
       const float4* gr = grads + warp * 32;
-#pragma unroll 8
-      for (int r = 0; r < 32; ++r) {
-        const uint32_t w2 = col[r * kRowWords];
-        const float hv = __uint_as_float((lane & 1) ? (w2 & 0xffff0000u) : (w2 << 16));
-        const float4 q = gr[r];
-        gw[0] += q.x * hv;
-        gw[1] += q.y * hv;
-        gw[2] += q.z * hv;
+      // pairwise over the 32 nodes, so that the running sum takes one rounding
+      // per 32 nodes, as many as when each thread summed its own nodes
+      float part[3] = {0.f, 0.f, 0.f};
+#pragma unroll 1
+      for (int r0 = 0; r0 < 32; r0 += 16) {
+        float s[2][3];
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+          float p[4][3];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int r = r0 + o * 8 + u * 2;
+            const uint32_t wa = col[r * kRowWords], wb = col[(r + 1) * kRowWords];
+            const float ha = __uint_as_float((lane & 1) ? (wa & 0xffff0000u) : (wa << 16));
+            const float hb = __uint_as_float((lane & 1) ? (wb & 0xffff0000u) : (wb << 16));
+            const float4 qa = gr[r], qb = gr[r + 1];
+            p[u][0] = fmaf(qb.x, hb, qa.x * ha);
+            p[u][1] = fmaf(qb.y, hb, qa.y * ha);
+            p[u][2] = fmaf(qb.z, hb, qa.z * ha);
+          }
+#pragma unroll
+          for (int m = 0; m < 3; ++m) s[o][m] = (p[0][m] + p[1][m]) + (p[2][m] + p[3][m]);
+        }
+#pragma unroll
+        for (int m = 0; m < 3; ++m) part[m] += s[0][m] + s[1][m];
       }
+#pragma unroll
+      for (int m = 0; m < 3; ++m) gw[m] += part[m];
       __syncwarp();
     }
   }
