@@ -1816,6 +1816,9 @@ sim_status sim_autotune(sim_h h, int n_steps, int* choices) {
     if (check_err(h, "sim_autotune") != SIM_OK) return 1e30;
     return t;
   };
+  // shapes of the separate adjoint kernels are scored on those, whatever the handle
+  // runs now; fused against separate comes after them
+  if (h->k > 0) h->tu.fuse_adjoint = 0;
   const int st_c[2] = {128, 256}, ga_c[3] = {128, 256, 512}, gb_c[3] = {1, 2, 4};
   double best = 1e30;
   int pick = h->tu.scatter_threads;
