@@ -177,7 +177,10 @@ advect_kernel(Geo g, const float4* __restrict__ pk, const uint8_t* __restrict__ 
 // FP64 adds for every cell would bound the two kernels below (GB300's FP64
 // rate is a small fraction of its FP32 rate): a thread sums in three FP32 words,
 // which loses nothing against FP64, and anew in FP64 where those overflow.
-constexpr int kSumPlanes = 16;  // planes along i a thread walks through
+// Planes along i a thread walks through: fewer FP64 sums with more of them, but a
+// small grid then has few threads, each waiting for its loads in turn (24^3: a pass
+// of one step and its adjoint 212 us with 16 planes, 202 with 4).
+__host__ __device__ inline int sum_planes(int n) { return n < 64 ? 4 : 16; }
 constexpr int kSumBatch = 8;    // of them loaded at a time
 
 // b = divergence of un on fluid cells (solid neighbours hold zero velocity);
@@ -186,7 +189,7 @@ __global__ void __launch_bounds__(kThreads)
 divergence_kernel(Geo g, const float* __restrict__ un, const uint8_t* __restrict__ nbr, float* __restrict__ b,
                   double* __restrict__ sum) {
   const int k = blockIdx.x * kBx + threadIdx.x, j = blockIdx.y * kBy + threadIdx.y;
-  const int i0 = blockIdx.z * kSumPlanes, i1 = min(i0 + kSumPlanes, g.n);
+  const int i0 = blockIdx.z * sum_planes(g.n), i1 = min(i0 + sum_planes(g.n), g.n);
   Sum3 acc;
   if (k < g.n && j < g.n) {
     const long long n1 = g.n, n2 = (long long)g.n * g.n, n3 = g.n3;
@@ -224,7 +227,7 @@ divergence_kernel(Geo g, const float* __restrict__ un, const uint8_t* __restrict
 __global__ void __launch_bounds__(kThreads)
 fluid_sum_kernel(Geo g, const float* __restrict__ x, const uint8_t* __restrict__ nbr, double* __restrict__ sum) {
   const int k = blockIdx.x * kBx + threadIdx.x, j = blockIdx.y * kBy + threadIdx.y;
-  const int i0 = blockIdx.z * kSumPlanes, i1 = min(i0 + kSumPlanes, g.n);
+  const int i0 = blockIdx.z * sum_planes(g.n), i1 = min(i0 + sum_planes(g.n), g.n);
   Sum3 acc;
   if (k < g.n && j < g.n) {
     for (int i = i0; i < i1; i += kSumBatch) {
@@ -735,7 +738,8 @@ struct mpm_gas {
   float* pack = nullptr;  // 4 n^3: packed fields (float4 per cell) of the step being advected
   double* sum = nullptr;
   float* mean = nullptr;
-  int* err = nullptr;  // set by a kernel whose bounded wait ran out
+  int* err = nullptr;   // set by a kernel whose bounded wait ran out
+  int* word = nullptr;  // pinned copy of err (grids whose sweeps go in pairs)
   int step = 0;
   bool started = false, seeds = false;
   long long launches = 0;
@@ -757,7 +761,9 @@ sim_status gcuda(gas_h h, cudaError_t e, const char* where) {
 
 inline int nblocks(long long m) { return int((m + kThreads - 1) / kThreads); }
 inline dim3 cell_grid(int n) { return dim3((n + kBx - 1) / kBx, (n + kBy - 1) / kBy, n); }
-inline dim3 sum_grid(int n) { return dim3((n + kBx - 1) / kBx, (n + kBy - 1) / kBy, (n + kSumPlanes - 1) / kSumPlanes); }
+inline dim3 sum_grid(int n) {
+  return dim3((n + kBx - 1) / kBx, (n + kBy - 1) / kBy, (n + sum_planes(n) - 1) / sum_planes(n));
+}
 const dim3 kCellBlock(kBx, kBy);
 
 // one Jacobi sweep, 4 cells a thread when n allows 16-byte rows
@@ -887,14 +893,17 @@ sim_status run_graph(gas_h h, std::vector<cudaGraphExec_t>& cache, std::vector<l
   return SIM_OK;
 }
 
+// Wait for the stream. Where sweeps go in pairs, whose waits are bounded, the error
+// word comes to pinned memory before it (to pageable memory, and for every solver, the
+// five calls of a 24^3 pass took 237 us instead of 205).
 sim_status sync(gas_h h, const char* where) {
-  int bad = 0;
-  cudaError_t e = cudaMemcpyAsync(&bad, h->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  cudaError_t e = cudaSuccess;
+  if (h->word) e = cudaMemcpyAsync(h->word, h->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
   const cudaError_t es = cudaStreamSynchronize(h->stream);
   if (e == cudaSuccess) e = es;
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return gcuda(h, e, where);
-  if (bad) {
+  if (h->word && *h->word) {
     cudaMemset(h->err, 0, sizeof(int));
     return gfail(h, SIM_E_TIMEOUT, std::string(where) + ": device wait timed out");
   }
@@ -942,9 +951,10 @@ sim_status gas_create(const gas_config* cfg, const uint8_t* solid, gas_h* out) {
   for (int q = 0; q < 8 && ok; ++q) ok = cudaMalloc(bufs[q], sizeof(float) * sizes[q]) == cudaSuccess;
   ok = ok && cudaMalloc(&h->sum, sizeof(double)) == cudaSuccess;
   ok = ok && cudaMalloc(&h->mean, sizeof(float)) == cudaSuccess;
-  ok = ok && cudaMalloc(&h->err, sizeof(int)) == cudaSuccess && cudaMemset(h->err, 0, sizeof(int)) == cudaSuccess;
   if (ok && n % 4 == 0 && n >= kPairFrom)
-    ok = cudaFuncSetAttribute(jacobi2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    ok = cudaMalloc(&h->err, sizeof(int)) == cudaSuccess && cudaMemset(h->err, 0, sizeof(int)) == cudaSuccess &&
+         cudaMallocHost(&h->word, sizeof(int)) == cudaSuccess &&
+         cudaFuncSetAttribute(jacobi2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               pair_smem_limit(h->sms)) == cudaSuccess;
   ok = ok && cudaMemcpy(h->solid, solid, n3, cudaMemcpyHostToDevice) == cudaSuccess;
   if (ok) {
@@ -975,6 +985,7 @@ sim_status gas_destroy(gas_h h) {
                     h->mean, h->pack, h->err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  if (h->word) cudaFreeHost(h->word);
   if (h->cstream) cudaStreamDestroy(h->cstream);
   delete h;
   return SIM_OK;
