@@ -705,13 +705,13 @@ finish_t_kernel(Geo g, const float4* __restrict__ acc, const uint8_t* __restrict
   dbar[c] = s ? 0.0f : a.w + g.beta_dt * a.y;
 }
 
-// zero `fields` consecutive n^3 fields of x on solid cells
+// zero a state's fields (u, d) on solid cells
 __global__ void __launch_bounds__(kThreads)
-mask_kernel(Geo g, const uint8_t* __restrict__ nbr, float* __restrict__ x, int fields) {
+mask_kernel(Geo g, const uint8_t* __restrict__ nbr, float* __restrict__ x) {
   int i, j, k;
   long long c;
   if (!my_cell(g.n, i, j, k, c) || !(nbr[c] & kSolidBit)) return;
-  for (int f = 0; f < fields; ++f) x[f * g.n3 + c] = 0.0f;
+  for (int f = 0; f < 4; ++f) x[f * g.n3 + c] = 0.0f;
 }
 
 __global__ void add_kernel(long long m, const float* __restrict__ a, float* __restrict__ b) {
@@ -999,7 +999,7 @@ sim_status gas_set_state(gas_h h, const float* u, const float* d, int on_device)
   cudaError_t e = copy_in(h, s0, u, sizeof(float) * 3 * n3, on_device);
   if (e == cudaSuccess) e = copy_in(h, s0 + 3 * n3, d, sizeof(float) * n3, on_device);
   if (e != cudaSuccess) return gcuda(h, e, "gas_set_state");
-  mask_kernel<<<cell_grid(h->g.n), kCellBlock, 0, h->stream>>>(h->g, h->nbr, s0, 4);
+  mask_kernel<<<cell_grid(h->g.n), kCellBlock, 0, h->stream>>>(h->g, h->nbr, s0);
   cudaMemsetAsync(h->adj, 0, sizeof(float) * 4 * n3, h->stream);
   h->launches += 1;
   h->step = 0;

@@ -279,19 +279,12 @@ void launch_sort(const Params& P, const float* st_in, const uint32_t* tag_in, co
 // ---------------------------------------------------------------------------
 // caller order <-> library order
 // ---------------------------------------------------------------------------
-// to_caller = 1: dst[pid[p] * fields + c] = src[c * stride_src + p]
-// to_caller = 0: dst[c * stride_dst + p] = src[pid[p] * fields + c]
-__global__ void gather_rows_kernel(const float* __restrict__ src, float* __restrict__ dst,
-                                   const int* __restrict__ pid, int N, int fields, int ss, int sd,
-                                   int to_caller) {
-  int p = blockIdx.x * blockDim.x + threadIdx.x;
+// rows of `fields` values -> SoA: dst[c * stride + p] = src[p * fields + c]
+__global__ void rows_to_fields_kernel(const float* __restrict__ src, float* __restrict__ dst, int N, int fields,
+                                      int stride) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= N) return;
-  long long q = pid ? pid[p] : p;
-  if (to_caller) {
-    for (int c = 0; c < fields; ++c) dst[q * fields + c] = src[(long long)c * ss + p];
-  } else {
-    for (int c = 0; c < fields; ++c) dst[(long long)c * sd + p] = src[q * fields + c];
-  }
+  for (int c = 0; c < fields; ++c) dst[(long long)c * stride + p] = src[(long long)p * fields + c];
 }
 
 __global__ void inverse_perm_kernel(const int* __restrict__ pid, int* __restrict__ inv, int N) {
@@ -321,11 +314,9 @@ void launch_permute_state(const float* src, float* dst, const int* pid_from, con
   permute_state_kernel<<<blocks_for(N, 256), 256, 0, s>>>(src, dst, inv, pid_to, N, n_first, f_first, fields);
 }
 
-void launch_gather_rows(const float* src, float* dst, const int* pid, int N, int fields,
-                        int field_stride_src, int field_stride_dst, int to_caller, cudaStream_t s) {
+void launch_rows_to_fields(const float* src, float* dst, int N, int fields, int stride, cudaStream_t s) {
   if (N == 0) return;
-  gather_rows_kernel<<<blocks_for(N, 256), 256, 0, s>>>(src, dst, pid, N, fields, field_stride_src,
-                                                       field_stride_dst, to_caller);
+  rows_to_fields_kernel<<<blocks_for(N, 256), 256, 0, s>>>(src, dst, N, fields, stride);
 }
 
 __global__ void init_state_kernel(float* __restrict__ st, int N) {

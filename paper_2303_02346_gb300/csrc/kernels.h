@@ -114,9 +114,8 @@ void launch_bin_clear(const Params& P, SortBuffers sb, cudaStream_t s);
 // water particles among the tags into *out (device int)
 void launch_count_water(const Params& P, const uint32_t* tag, int* out, cudaStream_t s);
 
-// permutations between the library's particle order and the caller's
-void launch_gather_rows(const float* src, float* dst, const int* pid, int N, int fields,
-                        int field_stride_src, int field_stride_dst, int to_caller, cudaStream_t s);
+// rows [N][fields] -> `fields` SoA fields of N values, `stride` apart
+void launch_rows_to_fields(const float* src, float* dst, int N, int fields, int stride, cudaStream_t s);
 
 // tool kinematics
 void launch_tool_forward(const Params& P, const float* pose0, const float* actions, int n_actions,

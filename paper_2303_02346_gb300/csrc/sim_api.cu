@@ -1150,7 +1150,7 @@ sim_status sim_set_state(sim_h h, int scene, const float* x, const float* v, con
     if (!src[f] || cnt == 0) continue;
     cudaError_t e = to_device(h, h->rows, src[f], sizeof(float) * 9 * cnt, on_device);
     if (e != cudaSuccess) return cuda_fail(h, e, "sim_set_state");
-    launch_gather_rows(h->rows, h->X0 + (size_t)(6 + 9 * f) * N + lo, nullptr, cnt, 9, 0, N, 0, h->stream);
+    launch_rows_to_fields(h->rows, h->X0 + (size_t)(6 + 9 * f) * N + lo, cnt, 9, N, h->stream);
     h->launches += 1;
   }
   restart(h);
