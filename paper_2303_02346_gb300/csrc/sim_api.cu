@@ -419,6 +419,10 @@ cudaError_t to_caller(sim_h h, void* dst, const void* src, size_t bytes, int on_
   return cudaStreamSynchronize(h->stream);
 }
 
+// Whether kernels can use a caller's device pointer as it is. Rows at any other
+// address go by copies, which take it.
+bool word_aligned(const void* p) { return reinterpret_cast<uintptr_t>(p) % sizeof(float) == 0; }
+
 bool scene_range(sim_h h, int scene, int* lo, int* cnt) {
   if (scene == -1) {
     *lo = 0;
@@ -1089,12 +1093,12 @@ sim_status sim_set_particles(sim_h h, int scene, const float* x, const float* v,
   const float *xs = x, *vs = v;
   const uint8_t* ms = mat;
   cudaError_t e = cudaSuccess;
-  if (!on_device) {
+  if (!on_device || !word_aligned(x) || !word_aligned(v)) {
     float* stage = h->rows;
     uint8_t* mstage = reinterpret_cast<uint8_t*>(stage + (size_t)6 * N);
-    e = to_device(h, stage, x, sizeof(float) * 3 * cnt, 0);
-    if (e == cudaSuccess) e = to_device(h, stage + (size_t)3 * N, v, sizeof(float) * 3 * cnt, 0);
-    if (e == cudaSuccess) e = to_device(h, mstage, mat, cnt, 0);
+    e = to_device(h, stage, x, sizeof(float) * 3 * cnt, on_device);
+    if (e == cudaSuccess) e = to_device(h, stage + (size_t)3 * N, v, sizeof(float) * 3 * cnt, on_device);
+    if (e == cudaSuccess) e = to_device(h, mstage, mat, cnt, on_device);
     if (e != cudaSuccess) return cuda_fail(h, e, "sim_set_particles");
     xs = stage;
     vs = stage + (size_t)3 * N;
@@ -1315,15 +1319,13 @@ sim_status sim_get_state(sim_h h, int scene, int step, float* x, float* v, float
   }
   // one pass from the state's own order to the caller's rows: straight into
   // device outputs, through the rows buffer for host ones
-  float* host[4] = {x, v, C, F};
+  float* outs[4] = {x, v, C, F};
   const int nc[4] = {3, 3, 9, 9};
   float* dev[4] = {x, v, C, F};
-  if (!on_device) {
-    size_t off = 0;
-    for (int q = 0; q < 4; ++q) {
-      dev[q] = host[q] ? h->rows + off : nullptr;
-      off += (size_t)nc[q] * cnt;
-    }
+  size_t off = 0;
+  for (int q = 0; q < 4; ++q) {
+    if (outs[q] && !(on_device && word_aligned(outs[q]))) dev[q] = h->rows + off;
+    off += (size_t)nc[q] * cnt;
   }
   cudaError_t e = cudaSuccess;
   if (on_device && h->stream) {
@@ -1339,9 +1341,10 @@ sim_status sim_get_state(sim_h h, int scene, int step, float* x, float* v, float
     h->launches += N > 0 && cnt > 0 ? 1 : 0;
   }
   e = cudaGetLastError();
-  for (int q = 0; q < 4 && !on_device && e == cudaSuccess; ++q)
-    if (host[q] && cnt)
-      e = cudaMemcpyAsync(host[q], dev[q], sizeof(float) * nc[q] * cnt, cudaMemcpyDeviceToHost, h->stream);
+  for (int q = 0; q < 4 && e == cudaSuccess; ++q)
+    if (outs[q] != dev[q] && cnt)
+      e = cudaMemcpyAsync(outs[q], dev[q], sizeof(float) * nc[q] * cnt,
+                          on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream);
   const cudaError_t es = cudaStreamSynchronize(h->stream);
   if (e == cudaSuccess) e = es;
   return e == cudaSuccess ? SIM_OK : cuda_fail(h, e, "sim_get_state");
@@ -1695,22 +1698,24 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
   h->rec_from = -1;  // the sweep's recomputes reuse the chunk buffers
   h->seeded.clear();   // the sweep added and cleared every pending seed
   // outputs in caller order, straight into device buffers, through the spare
-  // buffer for host ones; one wait for all of it. The sweep left the adjoint in
+  // buffer for others; one wait for all of it. The sweep left the adjoint in
   // `adj` or `rows` by its number of chunk boundaries (a replayed graph did not
   // run the swaps above).
   A = (nch_all - 1) % 2 ? h->rows : h->adj;
   spare = (nch_all - 1) % 2 ? h->adj : h->rows;
   cudaError_t e = cudaSuccess;
   if ((dLdx0 || dLdv0) && N > 0) {
-    float* host[2] = {dLdx0, dLdv0};
+    float* outs[2] = {dLdx0, dLdv0};
     float* dev[2] = {dLdx0, dLdv0};
-    for (int q = 0; q < 2 && !on_device; ++q) dev[q] = host[q] ? spare + (size_t)3 * q * N : nullptr;
+    for (int q = 0; q < 2; ++q)
+      if (outs[q] && !(on_device && word_aligned(outs[q]))) dev[q] = spare + (size_t)3 * q * N;
     launch_read_state(P, A, h->tag0, ck_pids(h, 0), 0, N, dev[0], dev[1], nullptr, nullptr, h->stream);
     h->launches += 1;
     e = cudaGetLastError();
-    for (int q = 0; q < 2 && !on_device && e == cudaSuccess; ++q)
-      if (host[q])
-        e = cudaMemcpyAsync(host[q], dev[q], sizeof(float) * 3 * N, cudaMemcpyDeviceToHost, h->stream);
+    for (int q = 0; q < 2 && e == cudaSuccess; ++q)
+      if (outs[q] != dev[q])
+        e = cudaMemcpyAsync(outs[q], dev[q], sizeof(float) * 3 * N,
+                            on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "sim_backward");
   }
   if (dLdactions && h->P.tool) {
