@@ -78,15 +78,16 @@ class Simulator:
         if self.scene.tool_enabled:
             self.set_tool()
 
-    def _empty(self, *shape):
-        """An output buffer of this shape. The library writes it on the handle's stream, but the allocator
-        orders its reuse by the current one, where work on the block's last owner may be pending: the
-        handle's stream waits for that. (The calls that fill outputs return when they are written.)"""
-        out = torch.empty(*shape, dtype=torch.float32, device=self.device)
-        current = torch.cuda.current_stream(self.device)
-        if current.cuda_stream != self.stream:
+    def _outputs(self, *shapes):
+        """Output buffers of these shapes. The library writes them on the handle's stream, but the allocator
+        orders a block's reuse by the current one, where work on its last owner may be pending: the
+        handle's stream waits for that. (The calls that fill outputs return when they are written.) The raw
+        handle is looked at first because making a Stream object takes some 7 us."""
+        outs = [torch.empty(*shape, dtype=torch.float32, device=self.device) for shape in shapes]
+        if torch._C._cuda_getCurrentRawStream(outs[0].get_device()) != self.stream:
+            current = torch.cuda.current_stream(self.device)
             torch.cuda.ExternalStream(self.stream, device=self.device).wait_stream(current)
-        return out
+        return outs
 
     # -- stepping and state -------------------------------------------------
     def step(self, n):
@@ -98,12 +99,9 @@ class Simulator:
 
     def state(self, scene=-1, with_CF=False, step=-1):
         cnt = self.N if scene < 0 else int(self.scene.scene_counts[scene])
-        x, v = self._empty(cnt, 3), self._empty(cnt, 3)
-        C = F = None
-        if with_CF:
-            C, F = self._empty(cnt, 3, 3), self._empty(cnt, 3, 3)
-        B.sim_get_state(self.h, scene, step, x, v, C, F)
-        return (x, v, C, F) if with_CF else (x, v)
+        outs = self._outputs(*[(cnt, 3)] * 2, *[(cnt, 3, 3)] * (2 if with_CF else 0))
+        B.sim_get_state(self.h, scene, step, *outs)
+        return tuple(outs)
 
     # -- losses and gradients -----------------------------------------------
     def position_loss(self, target, weight=1.0, scene=-1, step=-1):
@@ -122,7 +120,7 @@ class Simulator:
         dev = self.device
         e = torch.as_tensor(ell, dtype=torch.float32, device=dev).contiguous()
         gg = torch.as_tensor(g, dtype=torch.float32, device=dev).reshape(-1, 3).contiguous()
-        out = self._empty(*gg.shape)
+        out, = self._outputs(gg.shape)
         B.sim_share_gradients(self.h, scene, e, radius, tau, gg, out)
         return out
 
@@ -137,17 +135,16 @@ class Simulator:
     def tool_pose(self, step, scene=-1):
         """(S or 1, 13) tool pose at the start of `step`: position, quaternion
         (w, x, y, z), linear and angular velocity."""
-        out = self._empty(self.S if scene < 0 else 1, 13)
+        out, = self._outputs((self.S if scene < 0 else 1, 13))
         B.sim_get_tool_pose(self.h, scene, step, out)
         return out
 
     def backward(self, want_actions=True):
-        gx, gv = self._empty(self.N, 3), self._empty(self.N, 3)
-        ga = None
+        shapes = [(self.N, 3), (self.N, 3)]
         if want_actions and self.scene.tool_enabled:
             n_max = -(-self.max_steps // max(int(self.scene.substeps_per_action), 1))
-            n_act = min(self.scene.tool_actions.shape[-2], n_max)
-            ga = self._empty(self.S, n_act, 6)
+            shapes.append((self.S, min(self.scene.tool_actions.shape[-2], n_max), 6))
+        gx, gv, ga = (*self._outputs(*shapes), None)[:3]
         B.sim_backward(self.h, gx, gv, ga)
         return gx, gv, ga
 
