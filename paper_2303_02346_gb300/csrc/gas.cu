@@ -338,9 +338,10 @@ __device__ __forceinline__ Ends ends_of(bool first_in_row, bool last_in_row) {
 // cell), tab from fill_weights. p is zero on solid cells before and after every
 // sweep, so the sums need no tests; the bits matter only where a cell is solid
 // or misses a neighbour. A row's ends are told apart from other missing
-// neighbours because every warp holds one: testing each cell there made the
-// pair kernel's warps issue 438 instructions a plane, looking the weights up
-// 317, and with the ends set apart 291.
+// neighbours because every warp holds one. Instructions of a pair of sweeps over
+// 256^3 cells with an obstacle: 74.5 M (of warps) with each cell's bits tested
+// there, 54.0 M with the weights looked up, 49.5 M with the ends set apart (55.5 M
+// in a box of solid walls, where rows end in other bits).
 __device__ __forceinline__ float4 sweep4(const float4& P, const float4 (&Q)[4], float pl, float pr, const float4& R,
                                          uint32_t M4, const Ends& e, const float* tab, float h2) {
   float w[4] = {e.w0, 1.0f / 6.0f, 1.0f / 6.0f, e.w3}, out[4];
@@ -404,18 +405,18 @@ jacobi4_kernel(Geo g, const float* __restrict__ p_in, float* __restrict__ p_out,
 // through `seg` planes. A strip's rows of a plane are consecutive in memory, so
 // one bulk copy brings p (R + 2 rows) and one the right-hand side into a ring of
 // kStages planes, up to three planes ahead (~100 KB in flight per SM; with
-// plain loads one plane ahead the pair was no faster). At plane i the CTA sweeps its R rows once (i +- 1 in registers, j +- 1
-// from the ring), writes the result to a second ring of three planes, and
-// after the step's one barrier sweeps the inner R - 2 rows of plane i - 1 a
-// second time. The rows and planes of the halo are swept by both neighbours
-// ((R / (R - 2)) x ((seg + 2) / seg) of the first sweep's work, none of the
-// second's). Values are those of two single sweeps, bit for bit
-// (compared at 160^3 to 512^3). Every wait is bounded;
-// one that runs out sets *err. Measured per sweep (us, against one sweep a pass with
-// the same arithmetic; before it 5.4 / - / 20.6 / 40.1): 5.6 / 4.2 at 128^3, 8.9 /
-// 10.0 at 160^3, 13.4 / 17.0 at 192^3, 26.7 / 35.5 at 256^3: the pair is bound by
-// instruction issue (0.78 of the slots), the single sweep by DRAM, or by L2
-// where everything fits there.
+// plain loads one plane ahead the pair was no faster); the neighbour bits come by
+// plain loads, two planes ahead. At plane i the CTA sweeps its R rows once (i +- 1
+// in registers, j +- 1 from the ring), writes the result to a second ring of three
+// planes, and after the step's one barrier sweeps the inner R - 2 rows of plane
+// i - 1 a second time. The rows and planes of the halo are swept by both
+// neighbours ((R / (R - 2)) x ((seg + 2) / seg) of the first sweep's work, none of
+// the second's). Values are those of two single sweeps, bit for bit (compared at
+// 160^3 to 512^3). Every wait is bounded; one that runs out sets *err. Measured per
+// sweep (us, against one sweep a pass with the same arithmetic; before it 5.4 / - /
+// 20.6 / 40.1): 5.6 / 4.2 at 128^3, 8.9 / 10.0 at 160^3, 13.4 / 17.0 at 192^3, 26.7 /
+// 35.5 at 256^3: the pair is bound by instruction issue (0.82 of the slots), the
+// single sweep by DRAM, or by L2 where everything fits there.
 constexpr int kStages = 4;
 struct PairShape {
   int tx, rows, strips, seg, grid_i;

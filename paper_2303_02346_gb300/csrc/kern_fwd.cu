@@ -481,8 +481,9 @@ __device__ inline bool stage_gather_box(StageSmem<NT>& T, const Params& P, const
 // written once and scattered from registers without being read back (kLean:
 // only the part of it the next fused step reads; otherwise the 16 fields a
 // recomputed state keeps).
-// Registers as the compiler chooses them (80: 768 resident threads per SM)
-// or, with kHigh, held to 64 for 1024
+// Registers as the compiler chooses them (80 for the state-keeping step: 768
+// resident threads per SM; 104 for the lean one of 128 threads: 512) or, with
+// kHigh, held to 64 for 1024
 template <int NT, bool kExt, bool kLean, bool kStage, bool kHigh = false>
 __global__ void __launch_bounds__(NT, kHigh ? kScatterResidentThreadsHigh / NT : 0)
 g2p2g_kernel(Params P, const float* __restrict__ st_in, float* __restrict__ st_out,

@@ -30,7 +30,7 @@ static inline int blocks_for(long long n, int t) { return int((n + t - 1) / t); 
 // consecutive codes), the scan over the bins runs over the block counts, and
 // only the cells of blocks that hold particles are scanned, read and cleared
 // again; every bin and block count is zero between sorts. A re-sort of 2M
-// particles on 256^3: 366 -> 185 us, 133 of it the scatter of the state.
+// particles on 256^3: 366 -> 185 us so, about 140 with sort_gather_kernel.
 constexpr int kBlockBits = 6;  // cells of a 4^3 block: the lowest 6 bits of a code
 
 // One atomic per warp and cell (and per warp and block): the lanes of equal
@@ -436,7 +436,9 @@ int sm_count() {
 // * fused step and G2P adjoint at 8 resident CTAs (64 registers) against 6
 //   (80): 148 / 160 and 147 / 162 (2M), 45 / 47 and 46 / 50 (500k), 19.0 / 21.9
 //   and 17.7 / 22.1 (130k: one wave against two); 25.3 / 24.9 and 23.8 / 23.3
-//   (200k: two waves either way), 18.1 / 17.4 (100k: one wave either way).
+//   (200k: two waves either way), 18.1 / 17.4 (100k: one wave either way). The lean
+//   step of forward-only runs has 104 registers in the wide build, 4 CTAs, and was
+//   not measured apart.
 // * one adjoint kernel against two, whole reverse sweep: 0.53 / 0.74 ms (8k
 //   particles), 0.70 / 0.74 (100k), 1.86 / 1.90 (200k), 4.22 / 4.42 (500k), 7.85
 //   / 7.86 (1M), 15.1 / 14.7 (2M), 11.8 / 11.5 (3.2M in 64 scenes): fused saves a

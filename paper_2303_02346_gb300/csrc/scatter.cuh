@@ -39,9 +39,9 @@
 namespace mpm {
 
 constexpr int kRecF4 = 5;  // float4 per particle record: 4 used, the fifth keeps 16-byte stores free of bank conflicts
-// Resident threads per SM the scatter kernels are compiled for: 3 CTAs of 256
-// or 6 of 128 (at most 85 registers a thread) and, as a launch choice for the
-// fused step and the G2P adjoint, 4 CTAs of 256 or 8 of 128 (64 registers).
+// Resident threads per SM that the G2P adjoint is compiled for, 3 CTAs of 256 or 6 of
+// 128 (80 registers a thread; the fused step, left to the compiler, takes 80 to
+// 104), and, as a launch choice for both, 4 CTAs of 256 or 8 of 128 (64 registers).
 constexpr int kScatterResidentThreads = 768;
 constexpr int kScatterResidentThreadsHigh = 1024;
 
@@ -171,7 +171,10 @@ __device__ inline void warp_scatter(float4* rec, const Params& P, bool valid, in
       const float2 fxy = make_float2(r0.x, r0.y), fz = make_float2(r0.z, r0.z);
       const float2 wab = __ffma2_rn(__ffma2_rn(k2, fxy, k1), fxy, k0);  // (w_x(a), w_y(b))
       const float wxy = wab.x * wab.y;
-      // z weights of offsets 0 and 1; the third is 1 minus their sum
+      // z weights of offsets 0 and 1; the third is 1 minus their sum. f is a grid
+      // coordinate less a whole number, a multiple of 2^-22 from the third cell
+      // on: there the inner step is exact, and the polynomial is rounded once, to
+      // the very bits of the stencil's (1.5 - f)^2 / 2 and 3/4 - (f - 1)^2.
       const float2 wz = __ffma2_rn(__ffma2_rn(make_float2(0.5f, -1.0f), fz, make_float2(-1.5f, 2.0f)), fz,
                                    make_float2(1.125f, -0.25f));
       const float2 W01 = __fmul2_rn(make_float2(wxy, wxy), wz);
