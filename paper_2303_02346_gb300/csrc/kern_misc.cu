@@ -30,7 +30,8 @@ static inline int blocks_for(long long n, int t) { return int((n + t - 1) / t); 
 // consecutive codes), the scan over the bins runs over the block counts, and
 // only the cells of blocks that hold particles are scanned, read and cleared
 // again; every bin and block count is zero between sorts. A re-sort of 2M
-// particles on 256^3: 366 -> 185 us so, about 140 with sort_gather_kernel.
+// particles on 256^3: 366 -> 185 us so, 117 with sort_gather_kernel (mean of the 20
+// sorts of a trajectory, kernel by kernel).
 constexpr int kBlockBits = 6;  // cells of a 4^3 block: the lowest 6 bits of a code
 
 // One atomic per warp and cell (and per warp and block): the lanes of equal
