@@ -270,10 +270,10 @@ cudaError_t backward(sur_h h, int batch, const uint16_t* frames, const int* idx,
     Prof pr(h, "sur_proj");
     h->launches += 1;
     if (params)
-      e = launch_proj(h->g, batch, 2, frames, idx, tgt, h->h[h->B], h->params + po, h->params + po + 96, nullptr,
+      e = launch_proj(h->g, batch, h->num_sms, 2, frames, idx, tgt, h->h[h->B], h->params + po, h->params + po + 96, nullptr,
                       h->gh[0], g_frames ? h->gpred : nullptr, h->grad + po, h->dsum, nullptr, h->stream);
     else
-      e = launch_proj(h->g, batch, 8, frames, idx, nullptr, h->h[h->B], h->params + po, h->params + po + 96,
+      e = launch_proj(h->g, batch, h->num_sms, 8, frames, idx, nullptr, h->h[h->B], h->params + po, h->params + po + 96,
                       nullptr, h->gh[0], const_cast<float*>(g_pred_in), nullptr, nullptr, nullptr, h->stream);
   }
   int cur = 0;
@@ -498,7 +498,7 @@ sim_status sur_predict(sur_h h, int batch, const uint16_t* frames, const int* id
     Prof pr(h, "sur_proj");
     h->launches += 1;
     const long long po = proj_off(h->B);
-    e = launch_proj(h->g, batch, 1, frames, idx, nullptr, h->h[h->B], h->params + po, h->params + po + 96, pred,
+    e = launch_proj(h->g, batch, h->num_sms, 1, frames, idx, nullptr, h->h[h->B], h->params + po, h->params + po + 96, pred,
                     nullptr, nullptr, nullptr, nullptr, nullptr, h->stream);
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "sur_predict");
@@ -556,7 +556,7 @@ sim_status sur_eval(sur_h h, int batch, const uint16_t* frames, const int* idx, 
     Prof pr(h, "sur_proj");
     h->launches += 1;
     const long long po = proj_off(h->B);
-    e = launch_proj(h->g, batch, 4, frames, idx, tgt, h->h[h->B], h->params + po, h->params + po + 96, nullptr,
+    e = launch_proj(h->g, batch, h->num_sms, 4, frames, idx, tgt, h->h[h->B], h->params + po, h->params + po + 96, nullptr,
                     nullptr, nullptr, nullptr, nullptr, h->dsum + 1, h->stream);
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "sur_eval");

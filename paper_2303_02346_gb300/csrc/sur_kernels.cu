@@ -263,9 +263,11 @@ __device__ __forceinline__ void split_node(const SurGeom& g, long long v, int& i
 // ---------------------------------------------------------------------------
 // lift: h0 = bf16(W_l f + b_l) at every interior row. Memory moves 80 bytes a
 // node; the weights' shared-memory loads were the bound (one word per product),
-// so a thread takes two nodes and reads the weights 16 bytes at a time.
-// 8 frames of 64^3: 46 -> 39 us.
+// so a thread reads the weights 16 bytes at a time and, where there are more nodes
+// than threads, for two nodes (kTwo). 8 frames of 64^3: 46 -> 39 us; 3 frames of
+// 40^3, where the second node would be none: 13.2 -> 12.5 us (15.3 with kTwo).
 // ---------------------------------------------------------------------------
+template <bool kTwo>
 __global__ void __launch_bounds__(256) lift_kernel(SurGeom g, const uint16_t* __restrict__ frames,
                                                    const int* __restrict__ idx, const float* __restrict__ wl,
                                                    const float* __restrict__ bl, __nv_bfloat16* h0) {
@@ -277,9 +279,10 @@ __global__ void __launch_bounds__(256) lift_kernel(SurGeom g, const uint16_t* __
   const long long n3 = static_cast<long long>(g.n) * g.n * g.n;
   const long long fr = idx ? idx[b] : b;
   const long long step = static_cast<long long>(gridDim.x) * blockDim.x;
-  for (long long v0 = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; v0 < n3; v0 += 2 * step) {
+  for (long long v0 = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; v0 < n3;
+       v0 += (kTwo ? 2 : 1) * step) {
     const long long v1 = v0 + step;
-    const bool two = v1 < n3;
+    const bool two = kTwo && v1 < n3;
     const uint4 r0 = reinterpret_cast<const uint4*>(frames)[fr * n3 + v0];
     const uint4 r1 = two ? reinterpret_cast<const uint4*>(frames)[fr * n3 + v1] : r0;
     float f[2][8];
@@ -302,7 +305,7 @@ __global__ void __launch_bounds__(256) lift_kernel(SurGeom g, const uint16_t* __
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           s0 += w[q] * f[0][q];
-          s1 += w[q] * f[1][q];
+          if (kTwo) s1 += w[q] * f[1][q];
         }
         o0[e] = s0;
         o1[e] = s1;
@@ -644,16 +647,25 @@ cudaError_t launch_lift(const SurGeom& g, int batch, const uint16_t* frames, con
                         const float* b_lift, __nv_bfloat16* h0, cudaStream_t st) {
   const long long n3 = static_cast<long long>(g.n) * g.n * g.n;
   dim3 grid(static_cast<unsigned>(std::min<long long>((n3 + 255) / 256, 256)), batch);
-  lift_kernel<<<grid, 256, 0, st>>>(g, frames, idx, w_lift, b_lift, h0);
+  if (n3 > 256 * 256)
+    lift_kernel<true><<<grid, 256, 0, st>>>(g, frames, idx, w_lift, b_lift, h0);
+  else
+    lift_kernel<false><<<grid, 256, 0, st>>>(g, frames, idx, w_lift, b_lift, h0);
   return cudaGetLastError();
 }
 
-cudaError_t launch_proj(const SurGeom& g, int batch, int mode, const uint16_t* frames, const int* idx,
+// Nodes a thread walks through: 8 where parameter gradients are summed (fewer
+// atomics per entry). Elsewhere only as many as leave four CTAs for every SM: the
+// walk is a chain of loads (prediction of 3 frames of 40^3: 23.6 us with 8 nodes,
+// 12.3 with 2; of one frame of 24^3: 16.4 with 8, 8.0 with one).
+cudaError_t launch_proj(const SurGeom& g, int batch, int num_sms, int mode, const uint16_t* frames, const int* idx,
                         const int* tgt, const __nv_bfloat16* h, const float* w_proj, const float* b_proj,
                         float* pred, __nv_bfloat16* g_h, float* g_pred, float* grad_wp, double* loss_acc,
                         double* frame_sums, cudaStream_t st) {
   const long long n3 = static_cast<long long>(g.n) * g.n * g.n;
-  dim3 grid(static_cast<unsigned>(std::min<long long>((n3 + kProjThreads * 8 - 1) / (kProjThreads * 8), 512)),
+  const long long fill = 4LL * num_sms * kProjThreads;
+  const long long walk = (mode & 2) ? 8 : std::min<long long>(std::max<long long>((n3 * batch + fill - 1) / fill, 1), 8);
+  dim3 grid(static_cast<unsigned>(std::min<long long>((n3 + kProjThreads * walk - 1) / (kProjThreads * walk), 512)),
             batch);
   switch (mode) {
     case 1:

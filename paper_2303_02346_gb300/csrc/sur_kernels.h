@@ -94,7 +94,7 @@ cudaError_t launch_lift(const SurGeom& g, int batch, const uint16_t* frames, con
 // mode bit 1: write pred; bit 2: loss (*loss_acc += sum of squares) and
 // gradients; bit 4: per-frame error sums frame_sums[2b], [2b+1]; mode 8 alone:
 // dL/dh from a caller-supplied dL/dpred (g_pred, read)
-cudaError_t launch_proj(const SurGeom& g, int batch, int mode, const uint16_t* frames, const int* idx,
+cudaError_t launch_proj(const SurGeom& g, int batch, int num_sms, int mode, const uint16_t* frames, const int* idx,
                         const int* tgt, const __nv_bfloat16* h, const float* w_proj, const float* b_proj,
                         float* pred, __nv_bfloat16* g_h, float* g_pred, float* grad_wp, double* loss_acc,
                         double* frame_sums, cudaStream_t st);
