@@ -840,11 +840,10 @@ __device__ inline void block_add_double(double v, double* out) {
 // L_s = w sum |x - t|^2 over particles of scene `scene` (-1: all, per-scene
 // totals into loss[scene]); adj_x += 2 w (x - t). The FP64 units would bound it
 // (98 us at 2M particles with the sum in FP64 throughout, 17 us so), so a thread
-// sums the exact squares of its kLossItems particles in three FP32 words, which
+// sums the exact squares of its kItems particles in three FP32 words, which
 // loses nothing against FP64, and goes to FP64 once; particles are sorted by scene,
 // so its particles seldom belong to more than one loss entry, nor do a CTA's.
-constexpr int kLossItems = 8;
-
+template <int kItems>
 __global__ void __launch_bounds__(256)
 position_loss_kernel(Params P, const float* __restrict__ st, const uint32_t* __restrict__ tag,
                      int scene, float tx, float ty, float tz, float w,
@@ -852,15 +851,16 @@ position_loss_kernel(Params P, const float* __restrict__ st, const uint32_t* __r
   __shared__ double ws[8];
   __shared__ int wt[8];
   const int N = P.N;
-  const int base = blockIdx.x * (256 * kLossItems) + threadIdx.x;
+  constexpr int kBatch = 4;
+  const int base = blockIdx.x * (256 * kItems) + threadIdx.x;
   int cur = -1;
   Sum3 acc;
 #pragma unroll
-  for (int it = 0; it < kLossItems; it += 4) {
-    uint32_t tg[4];
-    float d[4][3], g[4][3];
+  for (int it = 0; it < kItems; it += kBatch) {
+    uint32_t tg[kBatch];
+    float d[kBatch][3], g[kBatch][3];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {  // all loads first; past the end: the last particle, not used
+    for (int u = 0; u < kBatch; ++u) {  // all loads first; past the end: the last particle, not used
       const int p = min(base + (it + u) * 256, N - 1);
       tg[u] = tag[p];
 #pragma unroll
@@ -870,7 +870,7 @@ position_loss_kernel(Params P, const float* __restrict__ st, const uint32_t* __r
       }
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < kBatch; ++u) {
       const int p = base + (it + u) * 256, sc = tag_scene(tg[u]);
       if (p >= N || (scene >= 0 && sc != scene)) continue;
       const float d0 = d[u][0] - tx, d1 = d[u][1] - ty, d2 = d[u][2] - tz;
@@ -926,11 +926,17 @@ position_loss_kernel(Params P, const float* __restrict__ st, const uint32_t* __r
   }
 }
 
+// Particles of a thread: with 8 the FP64 work is halved, with 4 the loads of a small
+// scene wait once (the whole call, us, 8 / 4: 34.5 / 29.8 at 3k particles, 36.4 / 29.7
+// at 100k, 38.1 / 38.2 at 500k, 39.5 / 50.3 at 2M).
+constexpr int kLossFour = 500000;
 void launch_position_loss(const Params& P, const float* st, const uint32_t* tag, int scene,
                           float tx, float ty, float tz, float w, float* adj, double* loss,
                           cudaStream_t s) {
   if (P.N == 0) return;
-  position_loss_kernel<<<blocks_for(P.N, 256 * kLossItems), 256, 0, s>>>(P, st, tag, scene, tx, ty, tz, w, adj, loss);
+  const int items = P.N < kLossFour ? 4 : 8;
+  auto k = items == 4 ? position_loss_kernel<4> : position_loss_kernel<8>;
+  k<<<blocks_for(P.N, 256 * items), 256, 0, s>>>(P, st, tag, scene, tx, ty, tz, w, adj, loss);
 }
 
 // P2G mass of the particles of one scene into a dense float grid

@@ -3,6 +3,7 @@ FP64's own rounding. All particles share one place, so that every thread's sum i
 off by the same amount and nothing averages out. Roundings on the way: one a
 thread's sum, one for the weight, five over a warp, eight over a CTA, one for the
 total: 16 of 2^-53 each, 1.8e-15, so 2e-15."""
+import math
 from fractions import Fraction
 
 import numpy as np
@@ -51,4 +52,24 @@ def test_target_met_and_nearly_met():
     near = np.array([np.nextafter(x[0, 0], np.float32(1)), x[0, 1], x[0, 2]], np.float32)
     want = _exact(x, near, 1.0)
     assert abs(Fraction(float(sim.position_loss(near)[0])) - want) <= want * Fraction(2e-15)
+    sim.close()
+
+
+def test_many_particles():
+    """Eight particles a thread (from 500,000 on): one more rounding for every CTA's
+    total, of 2048 particles."""
+    N = 600_001
+    n = 64
+    rng = np.random.default_rng(7)
+    sc = scenes.Scene(name="many", grid_n=n, dt=1e-4, n_steps=1, materials=[scenes.water_material((1.0 / n) ** 3 / 8)],
+                      x=0.2 + 0.6 * rng.random((N, 3)), v=np.zeros((N, 3)), mat=np.zeros(N, np.uint8), scene_counts=[N],
+                      checkpoint_every=1)
+    sim = Simulator(sc)
+    sim.reset()
+    sim.step(1)
+    target = np.array([0.4, 0.1, 0.9], np.float32)
+    d = (sim.state()[0].cpu().numpy() - target).astype(np.float64)
+    want = math.fsum((d * d).ravel())  # squares of FP32 numbers are exact in FP64
+    got = float(sim.position_loss(target)[0])
+    assert abs(got - want) <= want * (16 + N / 2048 + 1) * 2.0 ** -53
     sim.close()
