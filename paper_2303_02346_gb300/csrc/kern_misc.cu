@@ -140,7 +140,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_sums_kernel(uint32_t* __res
 
 // The cells of the occupied blocks: exclusive scan of each block's 64 counts
 // from the block's first slot, in place; blk_start receives that slot (the
-// scanned tile's value plus the tile's total). A warp looks at 32 blocks and
+// scanned tile's value plus the tiles' totals before it, sums; nullptr: there is
+// one tile). A warp looks at 32 blocks and
 // takes the occupied ones four at a time, 2 cells a lane, so that four blocks'
 // loads are in flight.
 __global__ void __launch_bounds__(256)
@@ -153,7 +154,7 @@ cell_scan_kernel(uint32_t* __restrict__ bins, const uint32_t* __restrict__ blk_c
   const bool occ = b < n_blk && blk_cnt[b] != 0u;
   uint32_t start = 0;
   if (occ) {
-    start = blk_start[b] + sums[b / kScanTile];
+    start = blk_start[b] + (sums ? sums[b / kScanTile] : 0u);
     blk_start[b] = start;
   }
   unsigned mask = __ballot_sync(kAll, occ);
@@ -232,20 +233,23 @@ sort_gather_kernel(int N, const float* __restrict__ st_in, const uint32_t* __res
   pid_out[q] = id;
 }
 
-static void bin_particles(const Params& P, const float* st, const uint32_t* tag, SortBuffers sb, int with_class,
+// Returns its launches.
+static int bin_particles(const Params& P, const float* st, const uint32_t* tag, SortBuffers sb, int with_class,
                           cudaStream_t s) {
   const int N = P.N;
-  if (N == 0) return;
+  if (N == 0) return 0;
   const int n_blk = int(((with_class ? 2LL : 1LL) * sb.n_bins) >> kBlockBits);
   sort_key_kernel<<<blocks_for(N, 256), 256, 0, s>>>(P, st, tag, sb.key, sb.rank, sb.bins, sb.blk_cnt, with_class);
   const int tiles = blocks_for(n_blk, kScanTile);
   scan_tiles_kernel<<<tiles, kScanThreads, 0, s>>>(sb.blk_cnt, sb.blk_start, n_blk, sb.tile_sums);
-  scan_sums_kernel<<<1, kScanThreads, 0, s>>>(sb.tile_sums, tiles);
-  cell_scan_kernel<<<blocks_for(n_blk, 256), 256, 0, s>>>(sb.bins, sb.blk_cnt, sb.blk_start, sb.tile_sums, n_blk);
+  if (tiles > 1) scan_sums_kernel<<<1, kScanThreads, 0, s>>>(sb.tile_sums, tiles);
+  cell_scan_kernel<<<blocks_for(n_blk, 256), 256, 0, s>>>(sb.bins, sb.blk_cnt, sb.blk_start,
+                                                          tiles > 1 ? sb.tile_sums : nullptr, n_blk);
+  return tiles > 1 ? 4 : 3;
 }
 
-void launch_bin(const Params& P, const float* st, const uint32_t* tag, SortBuffers sb, cudaStream_t s) {
-  bin_particles(P, st, tag, sb, 0, s);
+int launch_bin(const Params& P, const float* st, const uint32_t* tag, SortBuffers sb, cudaStream_t s) {
+  return bin_particles(P, st, tag, sb, 0, s);
 }
 
 void launch_bin_clear(const Params& P, SortBuffers sb, cudaStream_t s) {
@@ -267,14 +271,15 @@ void launch_count_water(const Params& P, const uint32_t* tag, int* out, cudaStre
   if (P.N > 0) count_water_kernel<<<blocks_for(P.N, 256), 256, 0, s>>>(P, tag, out);
 }
 
-void launch_sort(const Params& P, const float* st_in, const uint32_t* tag_in, const int* pid_in,
+int launch_sort(const Params& P, const float* st_in, const uint32_t* tag_in, const int* pid_in,
                  float* st_out, uint32_t* tag_out, int* pid_out, SortBuffers sb, cudaStream_t s) {
   const int N = P.N;
-  if (N == 0) return;
-  bin_particles(P, st_in, tag_in, sb, 1, s);
+  if (N == 0) return 0;
+  const int binned = bin_particles(P, st_in, tag_in, sb, 1, s);
   sort_index_kernel<<<blocks_for(N, 256), 256, 0, s>>>(N, sb.key, sb.rank, sb.bins, pid_out);
   sort_gather_kernel<<<blocks_for(N, 256), 256, 0, s>>>(N, st_in, tag_in, pid_in, st_out, tag_out, pid_out, P);
   launch_bin_clear(P, sb, s);
+  return binned + 3;
 }
 
 // ---------------------------------------------------------------------------

@@ -68,15 +68,18 @@ __device__ inline void for_candidates(const Params& P, int scene, const float4& 
         j0[z] = j1[z] = 0;
         if (cz < 0 || cz > P.n - 3) continue;
         const uint32_t k = kbase + morton3(uint32_t(cx), uint32_t(cy), uint32_t(cz));
-        // the block's count says whether its cells were scanned; its last cell
-        // ends where the block does
-        const uint32_t nb = __ldg(sb.blk_cnt + (k >> 6));
+        // a cell ends where the next one of its 4^3 block begins, the block's last
+        // one where the block does; blocks without particles hold zeros
         const uint32_t c0 = __ldg(sb.bins + k);
-        const uint32_t c1 = (k & 63u) == 63u ? __ldg(sb.blk_start + (k >> 6)) + nb : __ldg(sb.bins + k + 1);
-        if (nb) {
-          j0[z] = int(c0);
-          j1[z] = int(c1);
+        uint32_t c1;
+        if ((k & 63u) == 63u) {
+          const uint32_t nb = __ldg(sb.blk_cnt + (k >> 6));
+          c1 = nb ? __ldg(sb.blk_start + (k >> 6)) + nb : c0;
+        } else {
+          c1 = __ldg(sb.bins + k + 1);
         }
+        j0[z] = int(c0);
+        j1[z] = int(c1);
       }
 #pragma unroll
       for (int z = 0; z < 3; ++z)

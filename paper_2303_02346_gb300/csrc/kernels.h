@@ -106,8 +106,9 @@ struct SortBuffers {
   uint32_t* tile_sums;
   int n_bins;      // scenes x Morton codes per scene
 };
-// Sort by (class: water first, scene, Morton code of the stencil-origin cell)
-void launch_sort(const Params& P, const float* st_in, const uint32_t* tag_in, const int* pid_in,
+// Sort by (class: water first, scene, Morton code of the stencil-origin cell);
+// returns its launches
+int launch_sort(const Params& P, const float* st_in, const uint32_t* tag_in, const int* pid_in,
                  float* st_out, uint32_t* tag_out, int* pid_out, SortBuffers sb, cudaStream_t s);
 // Zero the bins and block counts that launch_bin (share.h) left for its readers
 void launch_bin_clear(const Params& P, SortBuffers sb, cudaStream_t s);

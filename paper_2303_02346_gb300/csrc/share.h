@@ -17,8 +17,8 @@ namespace mpm {
 // key of the 4^3 blocks that hold particles (64 consecutive keys, blk_cnt
 // nonzero; a key ends at the next one's first slot, a block's last key at
 // blk_start + blk_cnt). Uses the sort buffers; launch_bin_clear (kernels.h)
-// must follow the last kernel that reads them.
-void launch_bin(const Params& P, const float* st, const uint32_t* tag, SortBuffers sb, cudaStream_t s);
+// must follow the last kernel that reads them. Returns its launches.
+int launch_bin(const Params& P, const float* st, const uint32_t* tag, SortBuffers sb, cudaStream_t s);
 
 // Neighbour arrays in bin order. pk[slot] = (x, c) with c = exp(-ell[q] /
 // tau) for caller index q = pid[p] - lo in [0, cnt), else c = -1 (particle

@@ -379,8 +379,7 @@ void stage_rigid_adj(sim_h h, float* adj, const uint32_t* tag, const int* pid, c
 void do_sort(sim_h h, const float* st_in, const uint32_t* tag_in, const int* pid_in, float* st_out,
              uint32_t* tag_out, int* pid_out, cudaStream_t s) {
   Prof pr(h, "sort", s);
-  launch_sort(h->P, st_in, tag_in, pid_in, st_out, tag_out, pid_out, h->sb, s);
-  h->launches += h->P.N > 0 ? 7 : 0;
+  h->launches += launch_sort(h->P, st_in, tag_in, pid_in, st_out, tag_out, pid_out, h->sb, s);
 }
 
 // Wait for the stream and read the error word. The word is copied to pinned
@@ -1471,9 +1470,9 @@ static sim_status nbr_prepare(sim_h h, const char* where, int scene, const float
   cudaError_t e = to_device(h, s_ell, ell, sizeof(float) * (*cnt), on_device);
   if (e == cudaSuccess && g) e = to_device(h, s_g, g, sizeof(float) * 3 * (*cnt), on_device);
   if (e != cudaSuccess) return cuda_fail(h, e, where);
-  launch_bin(h->P, h->W, h->tag_cur, h->sb, h->stream);
+  h->launches += launch_bin(h->P, h->W, h->tag_cur, h->sb, h->stream);
   launch_nbr_pack(h->P, h->W, h->pid_cur, h->sb, s_ell, g ? s_g : nullptr, *lo, *cnt, tau, h->nb, h->stream);
-  h->launches += N > 0 ? 5 : 0;
+  h->launches += N > 0 ? 1 : 0;
   return SIM_OK;
 }
 

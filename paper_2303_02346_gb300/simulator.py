@@ -81,13 +81,16 @@ class Simulator:
     def _outputs(self, *shapes):
         """Output buffers of these shapes. The library writes them on the handle's stream, but the allocator
         orders a block's reuse by the current one, where work on its last owner may be pending: the
-        handle's stream waits for that. (The calls that fill outputs return when they are written.) The raw
-        handle is looked at first because making a Stream object takes some 7 us."""
-        outs = [torch.empty(*shape, dtype=torch.float32, device=self.device) for shape in shapes]
-        if torch._C._cuda_getCurrentRawStream(outs[0].get_device()) != self.stream:
-            current = torch.cuda.current_stream(self.device)
-            torch.cuda.ExternalStream(self.stream, device=self.device).wait_stream(current)
+        handle's stream waits for that. (The calls that fill outputs return when they are written.)"""
+        outs = [torch.empty(shape, dtype=torch.float32, device=self.device) for shape in shapes]
+        self._after_current(outs[0].get_device())
         return outs
+
+    def _after_current(self, device):
+        # the raw handle first: making a Stream object takes some 7 us
+        if torch._C._cuda_getCurrentRawStream(device) != self.stream:
+            current = torch.cuda.current_stream(device)
+            torch.cuda.ExternalStream(self.stream, device=device).wait_stream(current)
 
     # -- stepping and state -------------------------------------------------
     def step(self, n):
@@ -120,7 +123,8 @@ class Simulator:
         dev = self.device
         e = torch.as_tensor(ell, dtype=torch.float32, device=dev).contiguous()
         gg = torch.as_tensor(g, dtype=torch.float32, device=dev).reshape(-1, 3).contiguous()
-        out, = self._outputs(gg.shape)
+        out = torch.empty_like(gg)
+        self._after_current(out.get_device())
         B.sim_share_gradients(self.h, scene, e, radius, tau, gg, out)
         return out
 
