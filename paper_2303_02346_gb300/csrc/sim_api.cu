@@ -808,6 +808,12 @@ cudaGraphExec_t capture(sim_h h, Fn fn, bool node_priority = false) {
   return exec;
 }
 
+// After a capture failed: the handle's work is launched directly from now on,
+// unless an earlier error, still pending, is what kept the capture from starting.
+void no_graphs_from_now(sim_h h) {
+  if (cudaPeekAtLastError() == cudaSuccess) h->graphs = false;
+}
+
 // A checkpoint before the current step holds the state of step t = c*k
 // (c >= 1), in checkpoint c's particle order; false for any other step.
 bool retained_checkpoint(sim_h h, int t, int* c) {
@@ -1270,7 +1276,7 @@ static sim_status step_impl(sim_h h, int n_steps) {
     h->need_sort = ns;
     h->rec_from = lr;
     h->launches = l0;
-    h->graphs = false;
+    no_graphs_from_now(h);
     enqueue_steps(h, n_steps, h->stream);
     return check_err(h, "sim_step");
   }
@@ -1701,7 +1707,7 @@ sim_status sim_backward(sim_h h, float* dLdx0, float* dLdv0, float* dLdactions, 
         done = true;
       } else {
         h->launches = l0;
-        h->graphs = false;
+        no_graphs_from_now(h);
       }
     }
   }
